@@ -31,6 +31,7 @@ enum : int {
 struct EpiParams {
   int n_modes, n_det, n_phi;
   int mode_m[MAXM];
+  int kmode[MAXM];          // the mode whose azimuthal number is k + 1, or -1
   int npair;                // n_modes (n_modes - 1) / 2
   int pdelta[NPAIR];        // m_a - m_b of pair p (index into C_delta, 1..3)
   int consec;               // azimuthal numbers are consecutive: pdelta[p] = a - b

@@ -14,6 +14,14 @@
 // for y << 0), which leaves K small and smooth.  K is tabulated on a regular
 // (y, ln s) grid with its first and mixed derivatives (FP64 Gauss-Legendre,
 // built once per context) and read back by bicubic Hermite interpolation.
+//
+// The fused epilogues evaluate this for up to every phase of every pair, so the
+// usual range has a second table that holds everything but the dynamic range,
+//   R(y, ln s) = ln Lbar - (y >= 0 ? x^2 / 2 : s (x - s / 2)),
+// as one bicubic polynomial per cell (16 coefficients, 64 bytes, two 32-byte
+// loads): no erfc, no branches on y, 15 FMAs.  What bounds the uncut epilogue
+// is then the gather itself (32 different cells per warp), not the arithmetic.
+// Outside the cells' range the formula above is evaluated.
 #pragma once
 #include "common.cuh"
 
@@ -29,6 +37,17 @@ constexpr int DM_NY = DM_NA + DM_NB + DM_NC + 1;      // nodes
 constexpr float DM_S0 = -12.0f, DM_DS = 0.125f;
 constexpr int DM_NS = 145;
 constexpr float DM_HH_FLOOR = 1e-30f;
+
+// Cell table: ln s in [-6, 4) (step 1/8, the node grid's), y in [-64, 64): step 1/8 below
+// 0 and from 12 on, 1/16 on [0, 12) (there the peak sets in; measured against 64-bit
+// quadrature the cells are within 7e-6 of R at ln s = -10 and 1e-6 above ln s = 0, as the
+// node table is; median 5e-8).  Kept behind the node table in the same array.
+constexpr int DMC_N0 = 512, DMC_N1 = 192, DMC_N2 = 416;
+constexpr int DMC_NY = DMC_N0 + DMC_N1 + DMC_N2;
+constexpr float DMC_S0 = -6.0f, DMC_S1 = 4.0f;
+constexpr int DMC_NS = 80, DMC_IS0 = 48;  // ln s node DMC_IS0 of the node table is DMC_S0
+constexpr int DMC_OFF = (DM_NY * DM_NS + 3) / 4 * 4;  // first cell, in float4 units of the array
+constexpr int DM_TABLE_LEN = DMC_OFF + 4 * DMC_NY * DMC_NS;
 
 // node index -> y (host and device, exact in binary)
 __host__ __device__ __forceinline__ double dm_node_y(int iy) {
@@ -134,6 +153,75 @@ __device__ __forceinline__ float dm_lnlbar(float dh, float hh, float u_min, cons
   }
   const float C = 2.0175508218727822f;  // ln 3 + ln(2 pi)/2
   return base + C + 3.0f * sig - 4.0f * __logf(s + dm_mu(y)) + dm_table_K(y, sig, tab);
+}
+
+// Out-of-line: the cells' fallback, kept out of the hot loops' instruction stream.
+static __device__ __noinline__ float dm_lnlbar_call(float dh, float hh, float u_min, const float4 *tab) {
+  return dm_lnlbar(dh, hh, u_min, tab);
+}
+
+// One evaluation from the cells, in two steps so that a caller can have several
+// gathers in flight: the address and the cell coordinates, then the polynomial.
+struct DmCell {
+  float u, v, base;
+  bool in;  // inside the cells' range
+  const float4 *p;
+};
+
+__device__ __forceinline__ DmCell dm_cell_of(float dh, float hh, float u_min, const float4 *__restrict__ tab) {
+  DmCell c;
+  // 1 / sqrt(hh) to about an ulp: the approximation and one Newton step
+  const float q = rsqrt_ftz(hh);
+  const float t = hh * q;
+  const float ir = fmaf(0.5f * q, fmaf(-t, q, 1.0f), q);
+  const float x = dh * ir, s = u_min * (hh * ir);
+  const float y = x - s, sig = __logf(s);
+  c.base = (y >= 0.0f) ? 0.5f * x * x : s * fmaf(-0.5f, s, x);
+  c.in = hh > DM_HH_FLOOR && y >= -64.0f && y < 64.0f && sig >= DMC_S0 && sig < DMC_S1;
+  const bool fine = y >= 0.0f && y < 12.0f;
+  const float inv = fine ? 16.0f : 8.0f;
+  const float off = (y >= 12.0f) ? (float)(DMC_N0 + DMC_N1 - 96) : (float)DMC_N0;
+  const int iy = c.in ? min((int)fmaf(y, inv, off), DMC_NY - 1) : 0;
+  const int is = c.in ? min((int)fmaf(sig, 8.0f, -8.0f * DMC_S0), DMC_NS - 1) : 0;
+  c.u = fmaf(y, inv, off - (float)iy);
+  c.v = fmaf(sig, 8.0f, -8.0f * DMC_S0 - (float)is);
+  c.p = tab + DMC_OFF + 4 * (is * DMC_NY + iy);
+  return c;
+}
+
+__device__ __forceinline__ void ldg_nc8(const float4 *p, float (&a)[8]) {
+  asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=f"(a[0]), "=f"(a[1]), "=f"(a[2]), "=f"(a[3]), "=f"(a[4]), "=f"(a[5]), "=f"(a[6]), "=f"(a[7])
+               : "l"(p));
+}
+
+// R + base from the cell's coefficients a[l][k] of u^k v^l (l = 0, 1 in a, 2, 3 in b)
+__device__ __forceinline__ float dm_cell_value(const DmCell &c, const float (&a)[8], const float (&b)[8]) {
+  const float u = c.u, v = c.v;
+  const float c0 = fmaf(fmaf(fmaf(a[3], u, a[2]), u, a[1]), u, a[0]);
+  const float c1 = fmaf(fmaf(fmaf(a[7], u, a[6]), u, a[5]), u, a[4]);
+  const float c2 = fmaf(fmaf(fmaf(b[3], u, b[2]), u, b[1]), u, b[0]);
+  const float c3 = fmaf(fmaf(fmaf(b[7], u, b[6]), u, b[5]), u, b[4]);
+  return c.base + fmaf(fmaf(fmaf(c3, v, c2), v, c1), v, c0);
+}
+
+// ln Lbar(dh, hh) of N phases at once (their gathers overlap).
+template <int N>
+__device__ __forceinline__ void dm_lnlbar_n(const float (&dh)[N], const float (&hh)[N], float u_min,
+                                            const float4 *__restrict__ tab, float (&l)[N]) {
+  DmCell c[N];
+  float a[N][8], b[N][8];
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    c[k] = dm_cell_of(dh[k], hh[k], u_min, tab);
+    ldg_nc8(c[k].p, a[k]);
+    ldg_nc8(c[k].p + 2, b[k]);
+  }
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    l[k] = dm_cell_value(c[k], a[k], b[k]);
+    if (!c[k].in) l[k] = dm_lnlbar_call(dh[k], hh[k], u_min, tab);
+  }
 }
 
 }  // namespace dotpe

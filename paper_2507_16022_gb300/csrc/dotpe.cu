@@ -319,6 +319,8 @@ struct EventRun {
   TcWork W;
   ReduceArgs ra;
   bool mixed = false;
+  // the current block's <h|h> bound (tensor-core pass), for its screen and refinement
+  const __nv_bfloat16 *hmin = nullptr;
 };
 
 // The bank operand map and the shape common to every event of a launch.
@@ -404,6 +406,8 @@ static int event_alloc(dotpe_ctx *ctx, Event &e, cudaStream_t st, EventRun &R) {
   P.n_phi = e.nphi;
   P.n_pol = b.n_pol;
   for (int m = 0; m < MAXM; ++m) P.mode_m[m] = m < b.M ? b.mode_m[m] : 0;
+  for (int k = 0; k < MAXM; ++k) P.kmode[k] = -1;
+  for (int m = 0; m < b.M; ++m) P.kmode[b.mode_m[m] - 1] = m;
   P.npair = b.M * (b.M - 1) / 2;
   {
     int p = 0;
@@ -555,6 +559,8 @@ static EpiParams refine_params(const EventRun &R) {
   EpiParams Pf = R.P;
   Pf.ml_running = (float *)(R.scr + R.L.ml_refine);
   Pf.track_max = 0;
+  Pf.hmin = R.hmin;
+  Pf.hmin_ld = R.hmin ? hb_ld(R.P.n_ext) : 0;
   return Pf;
 }
 
@@ -589,6 +595,7 @@ static int hh_bound_pass(dotpe_ctx *ctx, const Event &e, EventRun &R, EpiParams 
   if (launch_hh_bound(R.P.n_int, e.NE, e.D, dl, R.P.mx, R.pa.qx, R.scr + R.L.hb, &hmin, ctx->n_sms, R.P.status,
                       st) != 0)
     return fail(DOTPE_E_DEVICE, "<h|h> bound launch failed: %s", cudaGetErrorString(cudaGetLastError()));
+  R.hmin = hmin;
   P.hmin = hmin;
   P.hmin_ld = hb_ld(e.NE);
   return DOTPE_OK;

@@ -275,7 +275,10 @@ __global__ void __launch_bounds__(SW * 32)
     dhh(k, dh, hh);
     const double ml = (dh > 0.0 && hh > 0.0) ? dh * dh / (2.0 * hh) : 0.0;
     if (!(ml >= a.threshold)) return (double)-INFINITY;
-    return (double)dm_lnlbar((float)dh, (float)hh, a.u_min, a.dm_table);
+    const float d1[1] = {(float)dh}, h1[1] = {(float)hh};
+    float l1[1];
+    dm_lnlbar_n<1>(d1, h1, a.u_min, a.dm_table, l1);
+    return (double)l1[0];
   });
   // ---- distance
   double dist = 0.0;

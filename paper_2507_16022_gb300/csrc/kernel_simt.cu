@@ -34,13 +34,14 @@ struct SimtSmem {
     SimtStage st[2];
     struct {
       float xs[TI][TE + 1], x2s[TI][TE + 1];
+      float z[8][2 * MAXM][NT];  // each thread's 8 pairs: (Re, Im) by azimuthal number
     } r;
   } u;
   float mls[TI][TE + 1];
   int pks[TI][TE + 1];  // argo | npass << 16
   alignas(16) float qs[TE * MAXD * REC];  // read as float4 records
   double lwe[TE];
-  float2 ph[7 * MAXPHI];
+  float4 ph[2 * MAXPHI];
   float r_m1[TI], r_s1[TI], r_m2[TI], r_s2[TI], r_ml[TI];
   long long r_arg[TI];
   int r_np[TI];
@@ -67,7 +68,7 @@ __global__ void __launch_bounds__(NT, 2) simt_fused_kernel(SimtArgs g, EpiParams
   auto &pks = S.pks;
   float *qs = S.qs;
   double *lwe = S.lwe;
-  float2 *ph = S.ph;
+  float4 *ph = S.ph;
   float *r_m1 = S.r_m1, *r_s1 = S.r_s1, *r_m2 = S.r_m2, *r_s2 = S.r_s2, *r_ml = S.r_ml;
   long long *r_arg = S.r_arg;
   int *r_np = S.r_np;
@@ -166,57 +167,65 @@ __global__ void __launch_bounds__(NT, 2) simt_fused_kernel(SimtArgs g, EpiParams
   const float thr = tile_threshold(P);
   const bool store = (P.lnl_tile != nullptr);
   const float zs = P.z_scale / (P.g_scale ? *P.g_scale : 1.f);
-  // epilogue: 4 rows x 2 extrinsic samples per thread
+  // epilogue: 4 rows x 2 extrinsic samples per thread, each thread's Z through its own
+  // column of shared memory (free after the mainloop), so that the pairs are a rolled loop
+  // and the accumulators' registers serve the evaluation
+  auto &zst = S.u.r.z;
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int rl = ty * 4 + r;
-    const int64_t i = i0 + rl;
-    const bool vi = i < P.n_int;
-    // the row's records are read through the cache for each pair (registers
-    // stay with the accumulators)
-    const bool pol = (P.n_pol == 2);
-    const float *mrow = P.mx + i * P.n_det * (pol ? REC_P : REC);
-    const double lwi = (vi && P.lw_int) ? P.lw_int[i] : 0.0;
+  for (int k = 0; k < MAXM; ++k) {
+    const int mk = P.kmode[k];  // (zero where the bank has no such mode)
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int el = tx + 16 * j;
-      const int64_t e = e0 + el;
-      float x = -INFINITY, x2 = -INFINITY, ml = -1.f;
-      int pk = 0;
-      if (vi && e < P.n_ext) {
-        float Zr[MAXM], Zi[MAXM];
+    for (int q = 0; q < 8; ++q)
 #pragma unroll
-        for (int mm = 0; mm < MAXM; ++mm) {
-          bool on = mm < P.n_modes;
-          Zr[mm] = on ? acc[mm][r][j][0] * zs : 0.f;
-          Zi[mm] = on ? acc[mm][r][j][1] * zs : 0.f;
-        }
-        if (P.gemm_only) {
-          float sx = 0.f;
+      for (int c = 0; c < 2; ++c) {
+        float v = 0.f;
 #pragma unroll
-          for (int mm = 0; mm < MAXM; ++mm) sx += Zr[mm] + Zi[mm];
-          x = sx; x2 = sx; ml = 0.f;
-        } else {
-          float C0, Cr[3], Ci[3];
-          if (pol) hh_coeffs_pol(mrow, &qs[el * MAXD * REC], P, C0, Cr, Ci);
-          else hh_coeffs<false>(mrow, &qs[el * MAXD * REC], P, C0, Cr, Ci);
-          PairRes pr = pair_eval(Zr, Zi, C0, Cr, Ci, thr, !store, P, ph);
-          float lw = (float)(lwi + lwe[el]);
-          x = pr.lsum + lw;
-          x2 = pr.lsum2 + 2.f * lw;
-          ml = pr.ml;
-          pk = pr.argo | (pr.npass << 16);
-          if (store) {
-            P.lnl_tile[i * P.n_ext + e] = pr.lsum - P.ln_nphi;
-            P.ml_tile[i * P.n_ext + e] = pr.ml;
-          }
+        for (int m = 0; m < MAXM; ++m) v = (m == mk) ? acc[m][q >> 1][q & 1][c] * zs : v;
+        zst[q][2 * k + c][tid] = v;
+      }
+  }
+  const bool pol = (P.n_pol == 2);
+#pragma unroll 1
+  for (int q = 0; q < 8; ++q) {
+    const int rl = ty * 4 + (q >> 1), el = tx + 16 * (q & 1);
+    const int64_t i = i0 + rl, e = e0 + el;
+    float x = -INFINITY, x2 = -INFINITY, ml = -1.f;
+    int pk = 0;
+    if (i < P.n_int && e < P.n_ext) {
+      // the row's records are read through the cache for each pair
+      const float *mrow = P.mx + i * P.n_det * (pol ? REC_P : REC);
+      const double lwi = P.lw_int ? P.lw_int[i] : 0.0;
+      float Zr[MAXM], Zi[MAXM];
+#pragma unroll
+      for (int k = 0; k < MAXM; ++k) {
+        Zr[k] = zst[q][2 * k][tid];
+        Zi[k] = zst[q][2 * k + 1][tid];
+      }
+      if (P.gemm_only) {
+        float sx = 0.f;
+#pragma unroll
+        for (int k = 0; k < MAXM; ++k) sx += Zr[k] + Zi[k];
+        x = sx; x2 = sx; ml = 0.f;
+      } else {
+        float C0, Cr[3], Ci[3];
+        if (pol) hh_coeffs_pol(mrow, &qs[el * MAXD * REC], P, C0, Cr, Ci);
+        else hh_coeffs_by<false>([&](int k) { return __ldg(mrow + k); }, &qs[el * MAXD * REC], P, C0, Cr, Ci);
+        PairRes pr = pair_eval(Zr, Zi, C0, Cr, Ci, thr, !store, P, ph);
+        float lw = (float)(lwi + lwe[el]);
+        x = pr.lsum + lw;
+        x2 = pr.lsum2 + 2.f * lw;
+        ml = pr.ml;
+        pk = pr.argo | (pr.npass << 16);
+        if (store) {
+          P.lnl_tile[i * P.n_ext + e] = pr.lsum - P.ln_nphi;
+          P.ml_tile[i * P.n_ext + e] = pr.ml;
         }
       }
-      xs[rl][el] = x;
-      x2s[rl][el] = x2;
-      mls[rl][el] = ml;
-      pks[rl][el] = pk;
     }
+    xs[rl][el] = x;
+    x2s[rl][el] = x2;
+    mls[rl][el] = ml;
+    pks[rl][el] = pk;
   }
   __syncthreads();
 

@@ -7,10 +7,10 @@
 //               k-blocks (one TMA transaction per operand and stage: the per-CTA
 //               TMA rate grows with the transaction size)
 //   warp 1      TMEM allocator and tcgen05.mma issuer (one elected lane)
-//   warps 2..9  epilogue (two warps per TMEM lane quadrant, each taking half
-//               of the tile's extrinsic samples): tcgen05.ld of the accumulators,
-//               <h|h> coefficients, phase grid, ML cut, distance marginal,
-//               log-sum-exp partials
+//   the others  epilogue, 8 warps (screens) or 16 (marginalisation): two or four per
+//               TMEM lane quadrant, each taking its share of the tile's extrinsic
+//               samples: tcgen05.ld of the accumulators, <h|h> coefficients, phase
+//               grid, ML cut, distance marginal, log-sum-exp partials
 // Tile = 128 bank rows x TEV extrinsic samples, all modes: accumulators for mode
 // m live in TMEM columns [buf * 4 * 2TEV + 2TEV m, +2TEV).  Per mode the GEMM is the
 // real-ified complex product of Eq. dh_ieo (K = 2B, padded to a multiple of 64).
@@ -51,9 +51,13 @@ namespace dotpe {
 
 namespace {
 constexpr int TI = TC_TI, TE = TC_TE, BK = 64;
-constexpr int NEPI = 8;              // epilogue warps
-constexpr int NT = (2 + NEPI) * 32;  // 320 threads
-constexpr int EPT = NEPI * 32;       // epilogue threads
+// Epilogue warps: 8 for the screens (168 registers, row records in registers), 16 for the
+// marginalising kernels (96 registers), whose table gathers and 32-phase loops are latency:
+// 12,289 rows x 771 samples without a cut (fp16x3) take 3.8 ms, 11.9 ms before with 8
+// warps, erfc / erfcx per phase and the node table; the refinement of 32,768 x 2,048
+// concentrated pairs 3.9 ms (5.2 ms), 2.85 ms of it its loads and MMAs alone.
+__host__ __device__ constexpr int epi_warps(int tev, bool scr) { return tev == 32 && !scr ? 16 : 8; }
+__host__ __device__ constexpr int cta_threads(int tev, bool scr) { return (2 + epi_warps(tev, scr)) * 32; }
 constexpr uint32_t A_BYTES = TI * BK * 2;  // one k-block of the bank tile
 constexpr int KBX = 2;  // k-blocks per stage (one 3-D TMA box)
 // Pipeline: single pass = 4 stages of {A, B} x 2 k-blocks (48 KB; 3 x 64 KB
@@ -74,22 +78,23 @@ constexpr uint32_t TMEM_COLS = 512;
 static_assert(2 * Pipe<false, 32>::BUF_COLS <= TMEM_COLS && Pipe<false, 64>::BUF_COLS <= TMEM_COLS, "TMEM budget");
 
 // TEV = 32 carries the general epilogue (marginalisation, partial sums through
-// shared memory); TEV = 64 only the screening and GEMM-only epilogues.
+// shared memory), or with SCR only its screen; TEV = 64 the screening and GEMM-only epilogues.
 constexpr int CAND_POOL = 32;  // candidate pairs per epilogue warp and 64-sample tile kept in shared memory
-template <int TEV> struct TcTail {
-  static constexpr bool GEN = (TEV == 32);
+constexpr int PAIR_POOL = 8;   // general epilogue: pairs per warp collected for an evaluation by 4 lanes each
+template <int TEV, bool SCR> struct TcTail {
+  static constexpr bool GEN = (TEV == 32 && !SCR);
+  static constexpr int NEPI = epi_warps(TEV, SCR);
   static constexpr int XS_LD = TEV + 1;
+  // pairs taken out of TMEM for a later evaluation: Z_m of every mode, and the owner lane and sample
+  static constexpr int POOL = TEV == 64 ? CAND_POOL : GEN ? PAIR_POOL : 0;
   EpiParams ep;  // parameters of the event whose tile the epilogue is on
-  float xs[GEN ? TI * XS_LD : 1];
+  float xs[TEV == 32 ? TI * XS_LD : 1];
   alignas(16) float qs[TEV * MAXD * REC];  // read as float4 records
   double lwe[GEN ? TEV : 1];
-  float2 ph[7 * MAXPHI];
-  float2 rowh[GEN ? TI : 1];  // second-half row partial of each row
+  float4 ph[2 * MAXPHI];
+  alignas(16) float pz[POOL ? NEPI * POOL * 2 * MAXM : 4];
+  int ptag[POOL ? NEPI * POOL : 1];
   float wm1[NEPI], ws1[NEPI], wm2[NEPI], ws2[NEPI], wml[NEPI];
-  // 64-sample screen: per-warp pool of candidate pairs taken out of TMEM
-  // (Z_m of every mode, and the owner lane and sample of the pair)
-  alignas(16) float pz[TEV == 64 ? NEPI * CAND_POOL * 2 * MAXM : 1];
-  int ptag[TEV == 64 ? NEPI * CAND_POOL : 1];
   long long warg[NEPI];
   int wnp[NEPI];
   uint64_t full[4], empty[4], tfull[2], tempty[2], drain;
@@ -97,12 +102,13 @@ template <int TEV> struct TcTail {
   uint32_t tmem_slot;
   int abort_flag;
 };
-template <bool SPLIT, int TEV, bool PAIR = false>
+template <bool SPLIT, int TEV, bool PAIR = false, bool SCR = false>
 constexpr size_t smem_bytes() {
-  return 1024 + (size_t)Pipe<SPLIT, TEV, PAIR>::ST * Pipe<SPLIT, TEV, PAIR>::STAGE + sizeof(TcTail<TEV>);
+  return 1024 + (size_t)Pipe<SPLIT, TEV, PAIR>::ST * Pipe<SPLIT, TEV, PAIR>::STAGE + sizeof(TcTail<TEV, SCR>);
 }
 static_assert(smem_bytes<true, 32>() <= 232448 && smem_bytes<false, 32>() <= 232448 &&
-                  smem_bytes<false, 64>() <= 232448 && smem_bytes<false, 64, true>() <= 232448,
+                  smem_bytes<false, 32, false, true>() <= 232448 && smem_bytes<false, 64>() <= 232448 &&
+                  smem_bytes<false, 64, true>() <= 232448,
               "shared memory budget");
 }  // namespace
 
@@ -196,19 +202,24 @@ __device__ __forceinline__ bool work_tile(const TcBatch<NB> &Bt, int w, int &k, 
 // M = 256): each CTA loads its own 128 bank rows and half of the tile's N
 // extrinsic rows, the even CTA issues the MMAs and commits them to both, and
 // each CTA's epilogue reads its own rows' accumulators from its own TMEM.
-template <bool BF16, int HH, bool SPLIT, int NB, bool SEP, int TEV, bool PAIR = false>
-__global__ void __launch_bounds__(NT, 1)
+// SCR (32-sample tiles): a screen that stores nothing per pair, without the marginalising
+// epilogue's code and its register needs.
+template <bool BF16, int HH, bool SPLIT, int NB, bool SEP, int TEV, bool PAIR = false, bool SCR = false>
+__global__ void __launch_bounds__(cta_threads(TEV, SCR), 1)
     tc_fused_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ TcBatch<NB> Bt,
                     const TcCommon C) {
   static_assert(SPLIT || !SEP, "a separate low-order accumulator needs split operands");
   static_assert(TEV == 32 || (TEV == 64 && !SPLIT && HH != 2), "64-sample tiles: single-pass mode banks");
   static_assert(!PAIR || (TEV == 64 && NB == 1), "CTA pairs: 64-sample tiles of one event");
   using PP = Pipe<SPLIT, TEV, PAIR>;
-  using TcTail = dotpe::TcTail<TEV>;
+  static_assert(!SCR || (TEV == 32 && !SPLIT), "screens: single pass");
+  using TcTail = dotpe::TcTail<TEV, SCR>;
+  constexpr int NEPI = TcTail::NEPI, EPT = NEPI * 32;  // epilogue warps and threads
   constexpr int ST = PP::ST, NPL = PP::NPL, BN = PP::BN;
   constexpr uint32_t STAGE_BYTES = PP::STAGE, A_ST = PP::A_ST, B_ST = PP::B_ST, B_BYTES = PP::B_BYTES;
   constexpr uint32_t BUF_COLS = PP::BUF_COLS;
-  constexpr int EHALF = TEV / 2;  // extrinsic samples per epilogue thread and tile
+  constexpr int NPART = NEPI / 4;      // epilogue warps per TMEM lane quadrant
+  constexpr int EHALF = TEV / NPART;   // extrinsic samples per epilogue thread and tile
   constexpr int XS_LD = TcTail::XS_LD;
   constexpr bool ONEBUF = SEP || TEV == 64;  // one accumulator set in flight
   constexpr int NUSE = SEP ? 2 : 1;           // accumulator uses per work tile (SEP: two 16-sample halves)
@@ -224,7 +235,13 @@ __global__ void __launch_bounds__(NT, 1)
   TcTail &T = *reinterpret_cast<TcTail *>(base + (size_t)ST * STAGE_BYTES);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int M = C.n_modes;
-  const int n_work = Bt.glist ? *Bt.glist_n : Bt.begin[Bt.n];
+  int n_work = Bt.glist ? *Bt.glist_n : Bt.begin[Bt.n];
+  if (Bt.gate) {
+    // no event of the launch takes this variant: nothing to walk
+    bool any = false;
+    for (int k = 0; k < Bt.n; ++k) any |= Bt.gate[k] == Bt.gate_want;
+    if (!any) n_work = 0;
+  }
   const int nst = (C.kb + KBX - 1) / KBX;  // stages per mode (an odd last k-block is zero-filled)
   const unsigned long long wait_ns = Bt.w[0].P.wait_ns;
   // work items: per CTA, or per CTA pair (consecutive blocks form a cluster)
@@ -413,10 +430,10 @@ __global__ void __launch_bounds__(NT, 1)
       mbar_wait(&T.drain, 0, nullptr, &no_abort, 500000000ull);
     }
   } else {
-    // ---------------- epilogue (256 threads: one tile row, half the samples each) ----------------
-    const int ew = warp - 2;      // 0..7
+    // ---------------- epilogue (one tile row and EHALF of its samples per thread) ----------------
+    const int ew = warp - 2;
     const int quad = warp & 3;    // TMEM lane quadrant this warp may access
-    const int half = ew >> 2;     // which 16 of the tile's 32 extrinsic samples
+    const int half = ew >> 2;     // which EHALF of the tile's extrinsic samples
     const int row = quad * 32 + lane;
     const int etid = threadIdx.x - 64;
     // one event: its parameters straight from kernel-parameter space (constant
@@ -427,7 +444,6 @@ __global__ void __launch_bounds__(NT, 1)
     constexpr int NREC = (HH == 2) ? POL_TC_MAXD * REC_POL : MAXD * REC;  // row record floats in registers
     float mrec[NREC];
 
-    double lwi = 0.0;
     int cur_it = -1, cur_k = -1;
     uint32_t u = 0;
     for (int w = w0; w < n_work; w += wstep) {
@@ -452,7 +468,6 @@ __global__ void __launch_bounds__(NT, 1)
         cur_k = k;
         cur_it = -1;
       }
-      const bool etv = true;
       const int t = it * Bt.w[k].n_etile + et;
       const int64_t i = (int64_t)it * TI + row;
       const bool vi = i < P.n_int;
@@ -489,8 +504,7 @@ __global__ void __launch_bounds__(NT, 1)
         }
       };
       if (it != cur_it) {
-        if constexpr (TEV == 32) load_mrec();
-        lwi = (vi && P.lw_int) ? P.lw_int[i] : 0.0;
+        if constexpr (SCR) load_mrec();
         cur_it = it;
       }
       // column records of the tile's samples, a float4 at a time (compile-time
@@ -542,6 +556,55 @@ __global__ void __launch_bounds__(NT, 1)
           }
         }
       }
+      // General epilogue.  With a cut and nothing stored a pair is skipped where an upper
+      // bound of its ln L^ML is below the threshold: the bound's <h|h> comes from the
+      // tensor-core pass where the event has it (the sum over modes is then all that a
+      // skipped pair costs), else from the pair's own coefficients.  Those, where every pair
+      // needs them, are formed here, while the tile's MMAs run, into a per-thread array.
+      bool skip = false, have_c = false;
+      float cf[TcTail::GEN ? EHALF : 1][8];
+      uint2 hw[2] = {make_uint2(0u, 0u), make_uint2(0u, 0u)};
+      if constexpr (TcTail::GEN) {
+        skip = thr > 0.f && !store && !P.gemm_only && !P.screen_ml;
+        have_c = !(skip && P.hmin) && !P.gemm_only;
+#pragma unroll
+        for (int j = 0; j < EHALF; ++j) T.xs[row * XS_LD + half * EHALF + j] = -INFINITY;
+        if (have_c) {
+          load_mrec();
+#pragma unroll 1
+          for (int j = 0; j < EHALF; ++j) {
+            const int el = SEP ? (16 * (j / (EHALF / 2)) + (EHALF / 2) * half + j % (EHALF / 2)) : (half * EHALF + j);
+            float C0, Cr[3], Ci[3];
+            hh_tile<HH>(mrec, &T.qs[el * MAXD * REC], P, C0, Cr, Ci);
+            float h = C0;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+              h -= 2.f * sqrt_up(Cr[q] * Cr[q] + Ci[q] * Ci[q]);
+              cf[j][1 + 2 * q] = Cr[q];
+              cf[j][2 + 2 * q] = Ci[q];
+            }
+            cf[j][0] = C0;
+            cf[j][7] = h;
+          }
+        } else if (skip) {
+          const int64_t ib = vi ? i : 0;
+          const __nv_bfloat16 *src = P.hmin + ib * P.hmin_ld + e0;
+#pragma unroll
+          for (int q = 0; q < 2; ++q)
+            hw[q] = __ldg(reinterpret_cast<const uint2 *>(src + (SEP ? 16 * q + 4 * half : EHALF * half + 4 * q)));
+        }
+      }
+      auto coef_of = [&](int j, float &C0, float (&Cr)[3], float (&Ci)[3]) {
+        C0 = cf[j][0];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) { Cr[q] = cf[j][1 + 2 * q]; Ci[q] = cf[j][2 + 2 * q]; }
+      };
+      auto hlow = [&](int j) -> float {
+        if (have_c) return cf[j][7];
+        const uint2 w2 = j < 4 ? hw[0] : hw[1];
+        const uint32_t w1 = (j & 2) ? w2.y : w2.x;
+        return __uint_as_float((j & 1) ? (w1 & 0xffff0000u) : (w1 << 16));
+      };
       // 64-sample screen with three or four modes: modes 0 and 1 complete first;
       // their share of sum_m |Z_m| per pair is read while the other modes' MMAs run
       const bool early = TEV == 64 && !P.gemm_only && M >= 3;
@@ -723,14 +786,15 @@ __global__ void __launch_bounds__(NT, 1)
                 hh_coeffs_by<HH == 1>([&](int q) { return __ldg(mrow + q); }, &T.qs[el * MAXD * REC], P, C0, Cr, Ci);
                 float Zr[MAXM], Zi[MAXM];
 #pragma unroll
-                for (int m = 0; m < MAXM; ++m) {
-                  if (m < M) {
+                for (int k = 0; k < MAXM; ++k) {
+                  const int m = P.kmode[k];
+                  if (m >= 0) {
                     const float2 z = *reinterpret_cast<const float2 *>(&pz[kk * 2 * MAXM + 2 * m]);
-                    Zr[m] = z.x * zs;
-                    Zi[m] = z.y * zs;
+                    Zr[k] = z.x * zs;
+                    Zi[k] = z.y * zs;
                   } else {
-                    Zr[m] = 0.f;
-                    Zi[m] = 0.f;
+                    Zr[k] = 0.f;
+                    Zi[k] = 0.f;
                   }
                 }
                 const float bound = pair_bound(Zr, Zi, C0, Cr, Ci);
@@ -817,14 +881,10 @@ __global__ void __launch_bounds__(NT, 1)
         continue;
       } else {
 
-      Lse ra, rb;
-      ra.init();
-      rb.init();
       float best = -1.f;
       long long barg = 0x7fffffffffffffffLL;
-      int np = 0;
       const uint32_t tbase = tmem + ((uint32_t)(quad * 32) << 16) + b * BUF_COLS;
-      if (!SPLIT && P.screen_ml && !store && !P.gemm_only) {
+      if constexpr (SCR) {
         // Screening without stored values needs only the tile's best ln L^ML.
         // Pass 1 bounds every pair of this thread (bounds kept in the thread's
         // own xs entries); pass 2 evaluates pairs in decreasing bound order
@@ -835,9 +895,10 @@ __global__ void __launch_bounds__(NT, 1)
           const int64_t e = e0 + half * EHALF + j;
           float Zr[MAXM], Zi[MAXM];
 #pragma unroll
-          for (int m = 0; m < MAXM; ++m) {
-            if (m < M) tmem_ld2(tbase + m * BN + 2 * (half * EHALF + j), Zr[m], Zi[m]);
-            else { Zr[m] = 0.f; Zi[m] = 0.f; }
+          for (int k = 0; k < MAXM; ++k) {
+            const int m = P.kmode[k];
+            if (m >= 0) tmem_ld2(tbase + m * BN + 2 * (half * EHALF + j), Zr[k], Zi[k]);
+            else { Zr[k] = 0.f; Zi[k] = 0.f; }
           }
           tmem_ld_wait();
           float bound = -INFINITY;
@@ -878,9 +939,10 @@ __global__ void __launch_bounds__(NT, 1)
             if (!__any_sync(0xffffffffu, want && jm == j)) continue;
             float zr[MAXM], zi[MAXM];
 #pragma unroll
-            for (int m = 0; m < MAXM; ++m) {
-              if (m < M) tmem_ld2(tbase + m * BN + 2 * (half * EHALF + j), zr[m], zi[m]);
-              else { zr[m] = 0.f; zi[m] = 0.f; }
+            for (int k = 0; k < MAXM; ++k) {
+              const int m = P.kmode[k];
+              if (m >= 0) tmem_ld2(tbase + m * BN + 2 * (half * EHALF + j), zr[k], zi[k]);
+              else { zr[k] = 0.f; zi[k] = 0.f; }
             }
             tmem_ld_wait();
             if (want && jm == j) {
@@ -944,156 +1006,260 @@ __global__ void __launch_bounds__(NT, 1)
         // of T.wml before any thread writes it again
         continue;
       } else {
+        // ---- marginalisation: the pairs of a 128 x 32 tile ----
+        Lse rb;
+        rb.init();
+        int np = 0;
+        auto sample_of = [&](int j) {
+          // SEP: samples of the first 16-sample half, then of the second
+          return SEP ? (16 * (j / (EHALF / 2)) + (EHALF / 2) * half + j % (EHALF / 2)) : (half * EHALF + j);
+        };
+        const float zcm = zs * zs * 1.000006f, thr2 = 2.f * thr;
+        const bool any_lw = P.lw_int || P.lw_ext;
+        float *pz = &T.pz[ew * PAIR_POOL * 2 * MAXM];
+        int *ptag = &T.ptag[ew * PAIR_POOL];
+        int npool = 0;  // warp-uniform
+        // One sample of each lane per step.  A pair that cannot reach the cut leaves no
+        // value.  Where more than PAIR_POOL of a step's 32 pairs are left, each lane
+        // evaluates its own; fewer are collected and evaluated PAIR_POOL at a time, four
+        // lanes to a pair (a quarter of the phases each), so that the phase grid is not
+        // walked by a warp for one or two of its lanes.
 #pragma unroll 1
-      for (int j = 0; j < EHALF; ++j) {
-        // SEP: samples of the first 16-sample half, then of the second (8 each)
-        const int el = SEP ? (16 * (j >> 3) + 8 * half + (j & 7)) : (half * EHALF + j);
-        const int64_t e = e0 + el;
-        float Zr[MAXM], Zi[MAXM];
-        if (SEP) {
-          if (j == 8) {
-            // the second half's accumulators
-            if (!mbar_wait(&T.tfull[b], (use + 1) & 1, nullptr, abortp, wait_ns)) break;
-            tc_fence_after();
-          }
-          // hi*hi in three interleaved sets, then the low-order set
-          const uint32_t col = tbase + 2 * (8 * half + (j & 7));
-          float Ar[4][MAXM], Ai[4][MAXM];
+        for (int j = 0; j <= EHALF; ++j) {
+          bool mine = false;
+          float Zr[MAXM], Zi[MAXM];
+          const int el = sample_of(min(j, EHALF - 1));
+          const int64_t e = e0 + el;
+          if (j < EHALF) {
+            if (SEP) {
+              if (j == EHALF / 2) {
+                // the second half's accumulators
+                if (!mbar_wait(&T.tfull[b], (use + 1) & 1, nullptr, abortp, wait_ns)) break;
+                tc_fence_after();
+              }
+              // hi*hi in three interleaved sets, then the low-order set
+              const uint32_t col = tbase + 2 * (el & 15);
+              float Ar[4][MAXM], Ai[4][MAXM];
 #pragma unroll
-          for (int qs = 0; qs < 4; ++qs)
+              for (int qs = 0; qs < 4; ++qs)
 #pragma unroll
-            for (int m = 0; m < MAXM; ++m) {
-              if (m < M) tmem_ld2(col + qs * SEP_SET + m * SEP_N, Ar[qs][m], Ai[qs][m]);
-              else { Ar[qs][m] = 0.f; Ai[qs][m] = 0.f; }
+                for (int k = 0; k < MAXM; ++k) {
+                  const int m = P.kmode[k];
+                  if (m >= 0) tmem_ld2(col + qs * SEP_SET + m * SEP_N, Ar[qs][k], Ai[qs][k]);
+                  else { Ar[qs][k] = 0.f; Ai[qs][k] = 0.f; }
+                }
+              tmem_ld_wait();
+#pragma unroll
+              for (int k = 0; k < MAXM; ++k) {
+                Zr[k] = ((Ar[0][k] + Ar[1][k]) + Ar[2][k]) + Ar[3][k];
+                Zi[k] = ((Ai[0][k] + Ai[1][k]) + Ai[2][k]) + Ai[3][k];
+              }
+            } else {
+#pragma unroll
+              for (int k = 0; k < MAXM; ++k) {
+                const int m = P.kmode[k];
+                if (m >= 0) tmem_ld2(tbase + m * BN + 2 * el, Zr[k], Zi[k]);
+                else { Zr[k] = 0.f; Zi[k] = 0.f; }
+              }
+              tmem_ld_wait();
             }
-          tmem_ld_wait();
+            if (j == EHALF - 1 || (SEP && j == EHALF / 2 - 1)) {
+              // this warp's accumulators are in registers: release the buffer to the MMA warp
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) release_acc(b);
+            }
+            mine = vi && e < P.n_ext;
+            if (skip) {
+              // |dh| <= sum |Z_m| against the lower bound of <h|h> at every phase
+              float a = 0.f;
 #pragma unroll
-          for (int m = 0; m < MAXM; ++m) {
-            Zr[m] = ((Ar[0][m] + Ar[1][m]) + Ar[2][m]) + Ar[3][m];
-            Zi[m] = ((Ai[0][m] + Ai[1][m]) + Ai[2][m]) + Ai[3][m];
-          }
-        } else {
+              for (int k = 0; k < MAXM; ++k) a += sqrt_near(fmaf(Zr[k], Zr[k], Zi[k] * Zi[k]));
+              const float h = hlow(j);
+              mine = mine && !(h > 0.f && zcm * a * a < thr2 * h);
+            }
 #pragma unroll
-          for (int m = 0; m < MAXM; ++m) {
-            if (m < M) tmem_ld2(tbase + m * BN + 2 * el, Zr[m], Zi[m]);
-            else { Zr[m] = 0.f; Zi[m] = 0.f; }
+            for (int k = 0; k < MAXM; ++k) {
+              Zr[k] *= zs;
+              Zi[k] *= zs;
+            }
           }
-          tmem_ld_wait();
-        }
-        if (j == EHALF - 1 || (SEP && j == 7)) {
-          // this warp's accumulators are in registers: release the buffer to the MMA warp
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) release_acc(b);
-        }
-        float x = -INFINITY, x2 = -INFINITY;
-        if (vi && e < P.n_ext) {
-#pragma unroll
-          for (int m = 0; m < MAXM; ++m) {
-            Zr[m] *= zs;
-            Zi[m] *= zs;
-          }
+          const uint32_t bal = __ballot_sync(0xffffffffu, mine);
+          const int cnt = __popc(bal);
+          const bool direct = cnt > 0 && (!skip || cnt > PAIR_POOL);
+          const bool flush = npool > 0 && (j == EHALF || (!direct && npool + cnt > PAIR_POOL));
           if (P.gemm_only) {
-            float sx = 0.f;
+            if (mine) {
+              float sx = 0.f;
 #pragma unroll
-            for (int m = 0; m < MAXM; ++m) sx += Zr[m] + Zi[m];
-            x = sx;
-            x2 = sx;
-          } else if (P.screen_ml) {
-            float C0, Cr[3], Ci[3];
-            hh_tile<HH>(mrec, &T.qs[el * MAXD * REC], P, C0, Cr, Ci);
-            int argo;
-            const float ml = pair_ml(Zr, Zi, C0, Cr, Ci, thr, !store, P, T.ph, argo);
-            if (ml > best) {
-              best = ml;
-              barg = (i * P.n_ext + e) * (long long)P.n_phi + argo;
+              for (int k = 0; k < MAXM; ++k) sx += Zr[k] + Zi[k];
+              T.xs[row * XS_LD + el] = sx;
+              rb.add(sx);
             }
-            if (store) {
-              P.lnl_tile[i * P.n_ext + e] = -INFINITY;
-              P.ml_tile[i * P.n_ext + e] = ml;
+            continue;
+          }
+          if (direct || flush) {
+            float zr[MAXM], zi[MAXM], C0, Cr[3], Ci[3];
+            bool act = mine;
+            int own = lane, sm = el;  // the pair: row of `own`, sample of the tile
+            if (!direct) {
+              __syncwarp();
+              const int kk = lane >> 2;
+              act = kk < npool;
+              const int tag = ptag[kk];
+              if (act) { own = tag >> 8; sm = tag & 255; }
+              const float4 *q4 = reinterpret_cast<const float4 *>(&pz[kk * 2 * MAXM]);
+              const float4 a = q4[0], c = q4[1];
+              zr[0] = a.x; zi[0] = a.y; zr[1] = a.z; zi[1] = a.w;
+              zr[2] = c.x; zi[2] = c.y; zr[3] = c.z; zi[3] = c.w;
+            } else {
+#pragma unroll
+              for (int k = 0; k < MAXM; ++k) { zr[k] = Zr[k]; zi[k] = Zi[k]; }
             }
-          } else {
-            float C0, Cr[3], Ci[3];
-            hh_tile<HH>(mrec, &T.qs[el * MAXD * REC], P, C0, Cr, Ci);
-            PairRes pr = pair_eval(Zr, Zi, C0, Cr, Ci, thr, !store, P, T.ph);
-            const float lw = (float)(lwi + T.lwe[el]);
-            x = pr.lsum + lw;
-            x2 = pr.lsum2 + 2.f * lw;
-            np += pr.npass;
-            if (pr.ml > best) {
-              best = pr.ml;
-              barg = (i * P.n_ext + e) * (long long)P.n_phi + pr.argo;
+            const int64_t io = (int64_t)it * TI + quad * 32 + own;
+            if (direct && have_c) {
+              coef_of(j, C0, Cr, Ci);
+            } else {
+              // from the row's record in memory; a collected pair's four lanes take a
+              // detector each and add (the order of the one-lane sum)
+              hh_row<HH>(P.mx, act ? io : (int64_t)0, &T.qs[sm * MAXD * REC], P, direct ? 0 : (lane & 3),
+                         direct ? P.n_det : min(P.n_det, (lane & 3) + 1), C0, Cr, Ci);
+              if (!direct) {
+#pragma unroll
+                for (int o = 1; o <= 2; o <<= 1) {
+                  C0 += __shfl_xor_sync(0xffffffffu, C0, o);
+#pragma unroll
+                  for (int k = 0; k < 3; ++k) {
+                    Cr[k] += __shfl_xor_sync(0xffffffffu, Cr[k], o);
+                    Ci[k] += __shfl_xor_sync(0xffffffffu, Ci[k], o);
+                  }
+                }
+              }
             }
-            if (store) {
-              P.lnl_tile[i * P.n_ext + e] = pr.lsum - P.ln_nphi;
-              P.ml_tile[i * P.n_ext + e] = pr.ml;
+            if (P.screen_ml) {
+              // (a screen that stores its pairs: best ln L^ML only)
+              if (act) {
+                int argo;
+                const float ml = pair_ml(zr, zi, C0, Cr, Ci, thr, false, P, T.ph, argo);
+                const long long g = (io * P.n_ext + e) * (long long)P.n_phi + argo;
+                if (ml > best || (ml == best && g < barg)) { best = ml; barg = g; }
+                if (store) {
+                  P.lnl_tile[i * P.n_ext + e] = -INFINITY;
+                  P.ml_tile[i * P.n_ext + e] = ml;
+                }
+              }
+              continue;
+            }
+            PhaseSums ps;
+            ps.init();
+            if (act) pair_phases(zr, zi, C0, Cr, Ci, thr, store, P, T.ph, direct ? 0 : (lane & 3), direct ? 1 : 4, ps);
+            if (!direct) {
+              ps.merge_xor(1);
+              ps.merge_xor(2);
+            }
+            if (act && (direct || (lane & 3) == 0)) {
+              const PairRes pr = ps.result();
+              float lw = 0.f;
+              if (any_lw) lw = (float)((P.lw_int ? P.lw_int[io] : 0.0) + T.lwe[sm]);
+              const float x = pr.lsum + lw;
+              T.xs[(quad * 32 + own) * XS_LD + sm] = x;
+              rb.add(pr.lsum2 + 2.f * lw);
+              np += pr.npass;
+              const long long g = (io * P.n_ext + e0 + sm) * (long long)P.n_phi + pr.argo;
+              if (pr.ml > best || (pr.ml == best && g < barg)) { best = pr.ml; barg = g; }
+              if (store) {
+                P.lnl_tile[io * P.n_ext + e0 + sm] = pr.lsum - P.ln_nphi;
+                P.ml_tile[io * P.n_ext + e0 + sm] = pr.ml;
+              }
+            }
+            if (!direct) {
+              npool = 0;
+              __syncwarp();
             }
           }
+          if (!direct && cnt > 0) {
+            const int slot = npool + __popc(bal & ((1u << lane) - 1u));
+            if (mine) {
+              ptag[slot] = (lane << 8) | el;
+              float4 *q4 = reinterpret_cast<float4 *>(&pz[slot * 2 * MAXM]);
+              q4[0] = make_float4(Zr[0], Zi[0], Zr[1], Zi[1]);
+              q4[1] = make_float4(Zr[2], Zi[2], Zr[3], Zi[3]);
+            }
+            npool += cnt;
+          }
         }
-        T.xs[row * XS_LD + el] = x;
-        ra.add(x);
-        rb.add(x2);
-      }
-      }
-      if (half == 1) T.rowh[row] = make_float2(ra.m, ra.s);
-      warp_merge_lse(rb);
-      warp_argmax(best, barg);
+        warp_merge_lse(rb);
+        warp_argmax(best, barg);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) np += __shfl_xor_sync(0xffffffffu, np, o);
-      {
-        Lse w = ra;
-        warp_merge_lse(w);
+        for (int o = 16; o > 0; o >>= 1) np += __shfl_xor_sync(0xffffffffu, np, o);
         if (lane == 0) {
-          T.wm1[ew] = w.m; T.ws1[ew] = w.s; T.wm2[ew] = rb.m; T.ws2[ew] = rb.s;
+          T.wm2[ew] = rb.m; T.ws2[ew] = rb.s;
           T.wml[ew] = best; T.warg[ew] = barg; T.wnp[ew] = np;
         }
-      }
-      named_bar_sync(1, EPT);
-      if (half == 0 && vi && etv) {
-        ra.merge(T.rowh[row].x, T.rowh[row].y);
-        P.row_part[(int64_t)et * P.n_int + i] = make_float2(ra.m, ra.s);
-      }
-      {
-        // column partials: 8 threads per extrinsic sample, 16 rows each
-        const int cc = etid >> 3, qq = etid & 7;
-        Lse a;
-        a.init();
-        for (int r = qq * 16; r < qq * 16 + 16; ++r) a.add(T.xs[r * XS_LD + cc]);
+        named_bar_sync(1, EPT);
+        {
+          // row partials: 4 threads per row, 8 samples each; their sum over the tile is its total
+          const int r = etid >> 2, q = etid & 3;
+          Lse a;
+          a.init();
 #pragma unroll
-        for (int o = 1; o <= 4; o <<= 1) {
-          float om = __shfl_xor_sync(0xffffffffu, a.m, o);
-          float os = __shfl_xor_sync(0xffffffffu, a.s, o);
-          a.merge(om, os);
-        }
-        if (qq == 0 && etv && e0 + cc < P.n_ext)
-          P.col_part[(int64_t)it * P.n_ext + e0 + cc] = make_float2(a.m, a.s);
-      }
-      if (etid < 32 && etv) {
-        // tile totals: lanes 0..NEPI-1 of the first epilogue warp hold the warps' values
-        Lse a, bb;
-        a.init();
-        bb.init();
-        float bv = -1.f;
-        long long bi = 0x7fffffffffffffffLL;
-        int n = 0;
-        if (etid < NEPI) {
-          a.merge(T.wm1[etid], T.ws1[etid]);
-          bb.merge(T.wm2[etid], T.ws2[etid]);
-          n = T.wnp[etid];
-          bv = T.wml[etid];
-          bi = T.warg[etid];
-        }
-        warp_merge_lse(a);
-        warp_merge_lse(bb);
-        warp_argmax(bv, bi);
+          for (int c = 0; c < TE / 4; ++c) a.add(T.xs[r * XS_LD + q * (TE / 4) + c]);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
-        if (etid == 0) {
-          P.tile_part[t] = make_float4(a.m, a.s, bb.m, bb.s);
-          P.tile_ml[t] = bv;
-          P.tile_arg[t] = bi;
-          P.tile_npass[t] = n;
-          if (bv > 0.f && P.track_max) atomic_max_nonneg(P.ml_running, bv);
+          for (int o = 1; o <= 2; o <<= 1) {
+            const float om = __shfl_xor_sync(0xffffffffu, a.m, o), os = __shfl_xor_sync(0xffffffffu, a.s, o);
+            a.merge(om, os);
+          }
+          const int64_t ir = (int64_t)it * TI + r;
+          if (q == 0 && ir < P.n_int) P.row_part[(int64_t)et * P.n_int + ir] = make_float2(a.m, a.s);
+#pragma unroll
+          for (int o = 4; o <= 16; o <<= 1) {
+            const float om = __shfl_xor_sync(0xffffffffu, a.m, o), os = __shfl_xor_sync(0xffffffffu, a.s, o);
+            a.merge(om, os);
+          }
+          if (lane == 0) { T.wm1[ew] = a.m; T.ws1[ew] = a.s; }
+        }
+        {
+          // column partials: 16 threads per extrinsic sample, every 16th row each
+          const int cc = etid >> 4, qq = etid & 15;
+          Lse a;
+          a.init();
+#pragma unroll
+          for (int r = 0; r < TI / 16; ++r) a.add(T.xs[(16 * r + qq) * XS_LD + cc]);
+#pragma unroll
+          for (int o = 1; o <= 8; o <<= 1) {
+            const float om = __shfl_xor_sync(0xffffffffu, a.m, o), os = __shfl_xor_sync(0xffffffffu, a.s, o);
+            a.merge(om, os);
+          }
+          if (qq == 0 && e0 + cc < P.n_ext) P.col_part[(int64_t)it * P.n_ext + e0 + cc] = make_float2(a.m, a.s);
+        }
+        named_bar_sync(1, EPT);
+        if (etid < 32) {
+          // tile totals: lanes 0..NEPI-1 of the first epilogue warp hold the warps' values
+          Lse a, bb;
+          a.init();
+          bb.init();
+          float bv = -1.f;
+          long long bi = 0x7fffffffffffffffLL;
+          int n = 0;
+          if (etid < NEPI) {
+            a.merge(T.wm1[etid], T.ws1[etid]);
+            bb.merge(T.wm2[etid], T.ws2[etid]);
+            n = T.wnp[etid];
+            bv = T.wml[etid];
+            bi = T.warg[etid];
+          }
+          warp_merge_lse(a);
+          warp_merge_lse(bb);
+          warp_argmax(bv, bi);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+          if (etid == 0) {
+            P.tile_part[t] = make_float4(a.m, a.s, bb.m, bb.s);
+            P.tile_ml[t] = bv;
+            P.tile_arg[t] = bi;
+            P.tile_npass[t] = n;
+            if (bv > 0.f && P.track_max) atomic_max_nonneg(P.ml_running, bv);
+          }
         }
       }
       // no trailing barrier: the next tile's barrier (after its column records)
@@ -1116,20 +1282,23 @@ __global__ void __launch_bounds__(NT, 1)
 
 // Launches one instantiation chosen by the run-time flags (the kernel's
 // parameter block is copied from *bt at launch).
-template <int NB, bool SPLIT, bool SEP, int TEV>
+template <int NB, bool SPLIT, bool SEP, int TEV, bool SCR = false>
 cudaError_t launch_tc_variant(const TcLaunch &L, const TcBatch<NB> &bt, int grid, cudaStream_t st) {
   auto go = [&](auto kern) -> cudaError_t {
-    const size_t smem = smem_bytes<SPLIT, TEV>();
+    const size_t smem = smem_bytes<SPLIT, TEV, false, SCR>();
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<grid, NT, smem, st>>>(L.mapA, bt, L.C);
+    kern<<<grid, cta_threads(TEV, SCR), smem, st>>>(L.mapA, bt, L.C);
     return cudaGetLastError();
   };
+  // screens are fp16 passes: no bf16 instantiation of SCR
+  constexpr bool BF = !SCR;
+  const bool bf16 = BF && L.bf16;
   if (L.pol) {
     // polarisation-resolved banks run one event per launch, in 32-sample tiles
     if constexpr (NB == 1 && TEV == 32)
-      return L.bf16 ? go(tc_fused_kernel<true, 2, SPLIT, NB, SEP, TEV>)
-                    : go(tc_fused_kernel<false, 2, SPLIT, NB, SEP, TEV>);
+      return bf16 ? go(tc_fused_kernel<BF, 2, SPLIT, NB, SEP, TEV, false, SCR>)
+                  : go(tc_fused_kernel<false, 2, SPLIT, NB, SEP, TEV, false, SCR>);
     else
       return cudaErrorInvalidValue;
   }
@@ -1142,7 +1311,7 @@ cudaError_t launch_tc_variant(const TcLaunch &L, const TcBatch<NB> &bt, int grid
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)grid, 1, 1);
-        cfg.blockDim = dim3(NT, 1, 1);
+        cfg.blockDim = dim3(cta_threads(64, false), 1, 1);
         cfg.dynamicSmemBytes = smem;
         cfg.stream = st;
         cudaLaunchAttribute at[1];
@@ -1175,10 +1344,10 @@ cudaError_t launch_tc_variant(const TcLaunch &L, const TcBatch<NB> &bt, int grid
                       : go2(tc_fused_kernel<false, 0, false, 1, false, 64, true>);
     }
   }
-  if (L.bf16) return L.consec ? go(tc_fused_kernel<true, 1, SPLIT, NB, SEP, TEV>)
-                              : go(tc_fused_kernel<true, 0, SPLIT, NB, SEP, TEV>);
-  return L.consec ? go(tc_fused_kernel<false, 1, SPLIT, NB, SEP, TEV>)
-                  : go(tc_fused_kernel<false, 0, SPLIT, NB, SEP, TEV>);
+  if (bf16) return L.consec ? go(tc_fused_kernel<BF, 1, SPLIT, NB, SEP, TEV, false, SCR>)
+                            : go(tc_fused_kernel<BF, 0, SPLIT, NB, SEP, TEV, false, SCR>);
+  return L.consec ? go(tc_fused_kernel<false, 1, SPLIT, NB, SEP, TEV, false, SCR>)
+                  : go(tc_fused_kernel<false, 0, SPLIT, NB, SEP, TEV, false, SCR>);
 }
 
 template <int NB>
@@ -1188,7 +1357,15 @@ cudaError_t launch_tc_any(const TcLaunch &L, const TcBatch<NB> &bt, int grid, cu
     if (L.split || L.pol || bt.glist) return cudaErrorInvalidValue;
     return launch_tc_variant<NB, false, false, 64>(L, bt, grid, st);
   }
-  if (!L.split) return launch_tc_variant<NB, false, false, 32>(L, bt, grid, st);
+  if (!L.split) {
+    bool scr = !L.bf16;
+    for (int k = 0; k < bt.n; ++k) {
+      const EpiParams &P = bt.w[k].P;
+      scr = scr && P.screen_ml && !P.lnl_tile && !P.gemm_only;
+    }
+    return scr ? launch_tc_variant<NB, false, false, 32, true>(L, bt, grid, st)
+               : launch_tc_variant<NB, false, false, 32>(L, bt, grid, st);
+  }
   return L.sep ? launch_tc_variant<NB, true, true, 32>(L, bt, grid, st)
                : launch_tc_variant<NB, true, false, 32>(L, bt, grid, st);
 }

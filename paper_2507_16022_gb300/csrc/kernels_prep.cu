@@ -622,10 +622,71 @@ __global__ void build_dm_table_kernel(float4 *__restrict__ tab) {
   tab[k] = make_float4((float)f, (float)fy, (float)(fs * DM_DS), (float)(fys * DM_DS));
 }
 
+// One cell of the polynomial table (see dist_marg.cuh): R and its derivatives at the
+// cell's four nodes, K's from the node table and the rest in closed form (FP64), then
+// the bicubic coefficients of u, v in [0, 1].
+__global__ void build_dm_cells_kernel(const float4 *__restrict__ tab, float4 *__restrict__ cells) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= DMC_NY * DMC_NS) return;
+  const int iy = k % DMC_NY, is = k / DMC_NY;
+  double F[4][4];  // rows: value at u = 0, 1, d/du at u = 0, 1; columns the same in v
+  for (int cy = 0; cy < 2; ++cy)
+    for (int cs = 0; cs < 2; ++cs) {
+      double y, hy;
+      if (iy < DMC_N0) { hy = 0.125; y = -64.0 + hy * (iy + cy); }
+      else if (iy < DMC_N0 + DMC_N1) { hy = 0.0625; y = hy * (iy - DMC_N0 + cy); }
+      else { hy = 0.125; y = 12.0 + hy * (iy - DMC_N0 - DMC_N1 + cy); }
+      int ny;  // the node table's index of y
+      if (y < -2.0) ny = (int)((y + 64.0) * 8.0 + 0.5);
+      else if (y < 12.0) ny = DM_NA + (int)((y + 2.0) * 32.0 + 0.5);
+      else ny = DM_NA + DM_NB + (int)((y - 12.0) * 8.0 + 0.5);
+      const int ns = DMC_IS0 + is + cs;
+      const float4 q = tab[ns * DM_NY + ny];
+      const double sig = (double)DM_S0 + (double)DM_DS * ns, s = exp(sig), m = mu_d(y);
+      const double dm = 0.5 * (1.0 + y / sqrt(y * y + 4.0));
+      // T = ln Phi(y) (+ y^2 / 2 on the side y < 0, whose base is s (x - s / 2))
+      double T, Ty;
+      if (iy < DMC_N0) {
+        const double ex = erfcx(-y * 0.70710678118654752);
+        T = log(0.5 * ex);
+        Ty = 0.79788456080286536 / ex + y;
+      } else {
+        const double Ph = 1.0 - 0.5 * erfc(y * 0.70710678118654752);
+        T = log(Ph);
+        Ty = 0.39894228040143268 * exp(-0.5 * y * y) / Ph;
+      }
+      const double C = 1.0986122886681098 + 0.91893853320467274;  // ln 3 + ln(2 pi) / 2
+      const double sm = s + m;
+      F[cy][cs] = (double)q.x + T + C + 3.0 * sig - 4.0 * log(sm);
+      F[2 + cy][cs] = hy * ((double)q.y + Ty - 4.0 * dm / sm);
+      F[cy][2 + cs] = (double)q.z + DM_DS * (3.0 - 4.0 * s / sm);
+      F[2 + cy][2 + cs] = hy * ((double)q.w + DM_DS * 4.0 * dm * s / (sm * sm));
+    }
+  // coefficients A = H F H^T of the Hermite basis
+  const double H[4][4] = {{1, 0, 0, 0}, {0, 0, 1, 0}, {-3, 3, -2, -1}, {2, -2, 1, 1}};
+  double P[4][4], A[4][4];
+  for (int a = 0; a < 4; ++a)
+    for (int j = 0; j < 4; ++j) {
+      P[a][j] = 0.0;
+      for (int t = 0; t < 4; ++t) P[a][j] += H[a][t] * F[t][j];
+    }
+  for (int a = 0; a < 4; ++a)
+    for (int l = 0; l < 4; ++l) {
+      A[a][l] = 0.0;
+      for (int t = 0; t < 4; ++t) A[a][l] += P[a][t] * H[l][t];
+    }
+  for (int l = 0; l < 4; ++l)
+    cells[4 * (int64_t)k + l] = make_float4((float)A[0][l], (float)A[1][l], (float)A[2][l], (float)A[3][l]);
+}
+
 __global__ void dist_marg_eval_kernel(int64_t n, const float *__restrict__ dh, const float *__restrict__ hh,
                                       float u_min, const float4 *__restrict__ tab, float *__restrict__ out) {
   int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (k < n) out[k] = dm_lnlbar(dh[k], hh[k], u_min, tab);
+  if (k >= n) return;
+  const float d[1] = {dh[k]}, h[1] = {hh[k]};
+  float l[1];
+  dm_lnlbar_n<1>(d, h, u_min, tab, l);
+  out[k] = l[0];
 }
 
 // ---------------------------------------------------------------------------
@@ -838,11 +899,11 @@ void launch_master_to_planes(int64_t n, const float *master, const float *amax, 
 }
 
 // The distance-marginal table is a constant of the method, the same for every
-// context: it lives in this static device array (3.2 MB, held by every GPU
+// context: it lives in this static device array (3.2 MB of nodes and 5.7 MB of cells, held by every GPU
 // that loads the library until the process exits) and is built once per CUDA
 // context of a device, by the first dotpe context created there, instead of
 // once per dotpe context.
-static __device__ __align__(256) float4 g_dm_table[DM_NY * DM_NS];
+static __device__ __align__(256) float4 g_dm_table[DM_TABLE_LEN];
 
 static unsigned long long current_ctx_id();
 
@@ -863,6 +924,7 @@ int shared_dm_table(int device, cudaStream_t st, float4 **tab, char *msg, size_t
     if (e == cudaSuccess && p == nullptr) e = cudaErrorInvalidSymbol;
     if (e == cudaSuccess) {
       build_dm_table_kernel<<<nblk((int64_t)DM_NY * DM_NS, 64), 64, 0, st>>>((float4 *)p);
+      build_dm_cells_kernel<<<nblk(DMC_NY * DMC_NS, 64), 64, 0, st>>>((const float4 *)p, (float4 *)p + DMC_OFF);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
