@@ -1562,7 +1562,8 @@ static int samples_locked(dotpe_ctx *ctx, Event &e, int64_t n, const double *uni
   if (!uniforms) return fail(DOTPE_E_INVALID, "null uniforms");
   cudaStream_t st = ctx->main_stream;
   Carver c;
-  const size_t o_u = c.take<double>((size_t)4 * n), o_cdf = c.take<double>(e.NI);
+  const size_t o_u = c.take<double>((size_t)4 * n), o_cdf = c.take<double>(sample_scratch_doubles(e.NI));
+  const size_t o_om = c.take<double>((size_t)e.D * b.B), o_cw = c.take<double2>((size_t)e.D * b.B);
   const size_t o_i = c.take<int64_t>(n), o_e = c.take<int64_t>(n), o_o = c.take<int32_t>(n), o_d = c.take<double>(n);
   const size_t o_st = c.take<int>(1);
   uint8_t *scr = nullptr;
@@ -1605,6 +1606,8 @@ static int samples_locked(dotpe_ctx *ctx, Event &e, int64_t n, const double *uni
   a.threshold = e.h_out->threshold;
   a.u_min = (float)e.u_min;
   a.dm_table = ctx->dm_table;
+  a.om = (double *)(scr + o_om);
+  a.cw = (double2 *)(scr + o_cw);
   a.status = (int *)(scr + o_st);
   if (rc == DOTPE_OK) {
     launch_sample(a, n, (const double *)(scr + o_u), (double *)(scr + o_cdf), (int64_t *)(scr + o_i),

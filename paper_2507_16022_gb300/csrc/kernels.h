@@ -341,10 +341,13 @@ struct SampleArgs {
   double threshold;             // the event's ML cut (-inf: none)
   float u_min;
   const float4 *dm_table;
+  double *om;                   // [D][B] scratch: 4 w / S (plain quadrature)
+  double2 *cw;                  // [D][B] scratch: 4 w conj(d) / S
   int *status;
 };
-// cdf: n_int doubles of scratch; outputs may be null
-void launch_sample(const SampleArgs &a, int64_t n, const double *uni, double *cdf, int64_t *i_out, int64_t *e_out,
+size_t sample_scratch_doubles(int64_t n_int);
+// scr: sample_scratch_doubles(n_int) doubles; outputs may be null
+void launch_sample(const SampleArgs &a, int64_t n, const double *uni, double *scr, int64_t *i_out, int64_t *e_out,
                    int32_t *o_out, double *d_out, cudaStream_t st);
 
 // Pilot tiles of a screening launch (cut on, grid order): a spread-out 1/48
