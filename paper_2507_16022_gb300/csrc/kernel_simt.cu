@@ -6,13 +6,21 @@
 // so each extrinsic sample e has two output columns, Re Z_m and Im Z_m.  The
 // FP32 extrinsic operand interleaves them along K, [m][e][Kpad][2].
 //
-// Mainloop: K in chunks of 16, every mode's A (64 bank rows) and B (32
-// samples) chunk copied into shared memory with cp.async (16-byte copies, two
-// stages: the next chunk's copies overlap this chunk's FMAs).  Each thread
-// accumulates 4 rows x 2 samples x (re, im) x 4 modes in registers; per k-quad
-// and mode it reads 4 + 4 float4 from shared memory for 64 FMAs (the A reads
-// are broadcasts, the B rows 36 words apart so that 16 lanes read 16 samples
-// in two wavefronts).
+// Mainloop: 64 threads per mode (a block has 64 n_modes), each with 8 rows x 4
+// samples of its mode in registers, (re, im) packed so that one instruction
+// (fma.rn.f32x2: both halves round as fmaf does) advances both.  K in chunks of 16 through two
+// cp.async stages that a mode's threads fill and order by a barrier of their own.  Per k-quad
+// a thread reads 8 + 8 times 16 bytes for 128 packed FMAs, every read one wavefront (rows 20
+// and samples 36 words apart), so shared memory is half busy and the FMA pipe is what is
+// left: 8,192 x 1,024, B 512, M 4 takes 2.6 ms without the epilogue (1.85 ms at the pipe's
+// rate), 2.8 ms with it and 3.1 ms with every pair stored.  It was 4.5 ms with every mode in each
+// thread (4 rows x 2 samples, shared memory 78% busy).  Measured and not kept: scalar FMAs
+// (3.7 ms), 4 rows x 8 samples (3.3 ms), sums split into even and odd k so that the
+// operands need no copy of the row's value into both halves (4 x 4 per thread, 3.7 ms).
+// The products of a pair are summed in k order.
+//
+// Epilogue: Z through shared memory (free after the mainloop), then a warp per row and a
+// lane per sample: the row's record is a broadcast, stored values are written in whole lines.
 #include "common.cuh"
 #include "epilogue.cuh"
 #include "kernels.h"
@@ -20,35 +28,31 @@
 namespace dotpe {
 
 namespace {
-constexpr int TI = SIMT_TI, TE = SIMT_TE, KC = 16, NT = 256;
+constexpr int TI = SIMT_TI, TE = SIMT_TE, KC = 16;
+constexpr int GT = 64;             // threads per mode
 constexpr int AS_LD = KC + 4;      // words per bank row of a stage
 constexpr int BS_LD = 2 * KC + 4;  // words per extrinsic sample of a stage ((re, im) per k)
-
-struct SimtStage {
-  float A[MAXM][TI][AS_LD];
-  float B[MAXM][TE][BS_LD];
-};
+constexpr int A_W = TI * AS_LD, B_W = TE * BS_LD;  // words of one mode's chunk
+constexpr int Z_W = TI * TE;                       // words of one component of Z
+constexpr int QS_LD = MAXD * REC + 4;  // words per column record: 16-byte reads of 8 lanes in 8 bank groups
+constexpr int MAXW = 2 * MAXM;         // warps of a block
+static_assert(2 * (A_W + B_W) >= 2 * Z_W, "Z fits in the stages");
 
 struct SimtSmem {
-  union {
-    SimtStage st[2];
-    struct {
-      float xs[TI][TE + 1], x2s[TI][TE + 1];
-      float z[8][2 * MAXM][NT];  // each thread's 8 pairs: (Re, Im) by azimuthal number
-    } r;
-  } u;
-  float mls[TI][TE + 1];
-  int pks[TI][TE + 1];  // argo | npass << 16
-  alignas(16) float qs[TE * MAXD * REC];  // read as float4 records
+  alignas(16) float qs[TE * QS_LD];
   double lwe[TE];
   float4 ph[2 * MAXPHI];
-  float r_m1[TI], r_s1[TI], r_m2[TI], r_s2[TI], r_ml[TI];
-  long long r_arg[TI];
-  int r_np[TI];
+  float2 col[MAXW][TE];                     // column partials of each warp's rows
+  float w_m1[MAXW], w_s1[MAXW], w_m2[MAXW], w_s2[MAXW], w_ml[MAXW];
+  long long w_arg[MAXW];
+  int w_np[MAXW];
 };
 
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem, bool valid) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(smem)), "l"(gmem),
+// the stages (or Z) of n_modes modes, then SimtSmem
+__host__ __device__ constexpr size_t stage_bytes(int n_modes) { return (size_t)n_modes * 2 * (A_W + B_W) * 4; }
+
+__device__ __forceinline__ void cp_async16(uint32_t smem, const void *gmem, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem), "l"(gmem),
                "r"(valid ? 16 : 0)
                : "memory");
 }
@@ -57,240 +61,218 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
+// c + a b for both halves of b and c
+__device__ __forceinline__ uint64_t fma2(float a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("{\n\t.reg .b64 t;\n\tmov.b64 t, {%1, %1};\n\tfma.rn.f32x2 %0, t, %2, %3;\n\t}"
+      : "=l"(d)
+      : "f"(a), "l"(b), "l"(c));
+  return d;
+}
+// Z of (component c, row, sample): eight samples of four consecutive rows in other banks
+__device__ __forceinline__ int z_at(int c, int row, int el) { return c * Z_W + row * TE + (el ^ ((row & 3) << 3)); }
 }  // namespace
 
-__global__ void __launch_bounds__(NT, 2) simt_fused_kernel(SimtArgs g, EpiParams P) {
+__global__ void __launch_bounds__(GT * MAXM, 2) simt_fused_kernel(SimtArgs g, EpiParams P) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
-  SimtSmem &S = *reinterpret_cast<SimtSmem *>(smem_raw);
-  auto &xs = S.u.r.xs;
-  auto &x2s = S.u.r.x2s;
-  auto &mls = S.mls;
-  auto &pks = S.pks;
-  float *qs = S.qs;
-  double *lwe = S.lwe;
-  float4 *ph = S.ph;
-  float *r_m1 = S.r_m1, *r_s1 = S.r_s1, *r_m2 = S.r_m2, *r_s2 = S.r_s2, *r_ml = S.r_ml;
-  long long *r_arg = S.r_arg;
-  int *r_np = S.r_np;
-
-  const int tid = threadIdx.x;
+  const int M = P.n_modes;
+  float *stage = reinterpret_cast<float *>(smem_raw);
+  SimtSmem &S = *reinterpret_cast<SimtSmem *>(smem_raw + stage_bytes(M));
+  const int tid = threadIdx.x, nt = blockDim.x;
   const int et = blockIdx.x, it = blockIdx.y;
   const int64_t i0 = (int64_t)it * TI, e0 = (int64_t)et * TE;
-  const int ty = tid / 16, tx = tid % 16;  // rows ty*4 .. ty*4+3, samples tx and tx + 16
-  const int M = P.n_modes;
+  const int m = tid / GT, t = tid % GT;  // this thread's mode
+  const int ty = t / 8, tx = t % 8;      // rows ty + 8 r, samples tx + 8 j
 
-  fill_phase_tables(ph, P, tid, NT);
-  for (int k = tid; k < TE * P.n_det * REC; k += NT) {
-    int e = k / (P.n_det * REC), q = k % (P.n_det * REC);
-    qs[e * MAXD * REC + q] = (e0 + e < P.n_ext) ? P.qx[(e0 + e) * P.n_det * REC + q] : 0.f;
+  fill_phase_tables(S.ph, P, tid, nt);
+  for (int k = tid; k < TE * P.n_det * REC; k += nt) {
+    const int e = k / (P.n_det * REC), q = k % (P.n_det * REC);
+    S.qs[e * QS_LD + q] = (e0 + e < P.n_ext) ? P.qx[(e0 + e) * P.n_det * REC + q] : 0.f;
   }
-  for (int k = tid; k < TE; k += NT) lwe[k] = (P.lw_ext && e0 + k < P.n_ext) ? P.lw_ext[e0 + k] : 0.0;
+  for (int k = tid; k < TE; k += nt) S.lwe[k] = (P.lw_ext && e0 + k < P.n_ext) ? P.lw_ext[e0 + k] : 0.0;
 
-  float acc[MAXM][4][2][2];
+  // (re, im) packed: one instruction adds both (each half rounds as fmaf does)
+  uint64_t acc[8][4];
 #pragma unroll
-  for (int m = 0; m < MAXM; ++m)
+  for (int r = 0; r < 8; ++r)
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        acc[m][r][j][0] = 0.f;
-        acc[m][r][j][1] = 0.f;
-      }
+    for (int j = 0; j < 4; ++j) acc[r][j] = 0ull;
 
-  // one chunk of every mode's operands into stage s (zero-filled outside the
-  // slice, the extrinsic samples and the modes)
+  // one chunk of this mode's operands into stage s (zero-filled outside the
+  // slice and the extrinsic samples)
   const int nch = (g.K + KC - 1) / KC;
-  auto load_chunk = [&](int c, int s) {
-    const int k0 = c * KC;
-    SimtStage &st = S.u.st[s];
-    for (int f = tid; f < MAXM * TI * (KC / 4); f += NT) {
-      const int m = f / (TI * (KC / 4)), r = (f / (KC / 4)) % TI, q = f % (KC / 4);
-      const bool ok = m < M && i0 + r < P.n_int;
-      const float *src = ok ? g.A + ((int64_t)m * g.I_bank + P.i_base + i0 + r) * g.Kpad + k0 + 4 * q : g.A;
-      cp_async16(&st.A[m][r][4 * q], src, ok);
-    }
-    for (int f = tid; f < MAXM * TE * (2 * KC / 4); f += NT) {
-      const int m = f / (TE * (2 * KC / 4)), e = (f / (2 * KC / 4)) % TE, q = f % (2 * KC / 4);
-      const bool ok = m < M && e0 + e < P.n_ext;
-      const float *src = ok ? g.Bm + (((int64_t)m * P.n_ext + e0 + e) * g.Kpad + k0) * 2 + 4 * q : g.Bm;
-      cp_async16(&st.B[m][e][4 * q], src, ok);
-    }
+  // (a thread's copies: 16 bytes of rows t / 4 + 16 p and of samples t / 8 + 8 p, p = 0..3;
+  // pointers, strides and the in-range bits are set up once)
+  const float *ap = g.A + ((int64_t)m * g.I_bank + P.i_base + i0 + t / 4) * g.Kpad + 4 * (t % 4);
+  const float *bp = g.Bm + (((int64_t)m * P.n_ext + e0 + t / 8) * g.Kpad) * 2 + 4 * (t % 8);
+  uint32_t inb = 0;
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    inb |= (i0 + t / 4 + 16 * p < P.n_int) ? 1u << p : 0u;
+    inb |= (e0 + t / 8 + 8 * p < P.n_ext) ? 16u << p : 0u;
+  }
+  const uint32_t sdst = smem_u32(stage + m * 2 * (A_W + B_W)) + 4 * (t / 4 * AS_LD + 4 * (t % 4));
+  const uint32_t tdst = smem_u32(stage + m * 2 * (A_W + B_W) + A_W) + 4 * (t / 8 * BS_LD + 4 * (t % 8));
+  const int astep = 16 * g.Kpad, bstep = 16 * g.Kpad;
+  auto load_chunk = [&](int s) {
+    const uint32_t so = s * (A_W + B_W) * 4;
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+      cp_async16(sdst + so + p * 16 * AS_LD * 4, (inb >> p) & 1 ? ap + p * astep : g.A, (inb >> p) & 1);
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+      cp_async16(tdst + so + p * 8 * BS_LD * 4, (inb >> (4 + p)) & 1 ? bp + p * bstep : g.Bm, (inb >> (4 + p)) & 1);
     cp_async_commit();
+    ap += KC;
+    bp += 2 * KC;
   };
 
-  load_chunk(0, 0);
+  load_chunk(0);
 #pragma unroll 1
   for (int c = 0; c < nch; ++c) {
     if (c + 1 < nch) {
-      load_chunk(c + 1, (c + 1) & 1);
+      load_chunk((c + 1) & 1);
       cp_async_wait<1>();
     } else {
       cp_async_wait<0>();
     }
-    __syncthreads();
-    const SimtStage &st = S.u.st[c & 1];
+    named_bar_sync(1 + m, GT);
+    const float *A = stage + (m * 2 + (c & 1)) * (A_W + B_W), *B = A + A_W;
 #pragma unroll
-    for (int m = 0; m < MAXM; ++m) {
-      if (m >= M) break;
+    for (int kq = 0; kq < KC / 4; ++kq) {
+      float4 a[8];
 #pragma unroll
-      for (int kq = 0; kq < KC / 4; ++kq) {
-        float4 a[4], b[2][2];
+      for (int r = 0; r < 8; ++r) a[r] = *reinterpret_cast<const float4 *>(A + (ty + 8 * r) * AS_LD + 4 * kq);
 #pragma unroll
-        for (int r = 0; r < 4; ++r) a[r] = *reinterpret_cast<const float4 *>(&st.A[m][ty * 4 + r][4 * kq]);
+      for (int j = 0; j < 4; ++j) {
+        // (re, im) of k, k+1 and of k+2, k+3
+        const ulonglong2 b0 = *reinterpret_cast<const ulonglong2 *>(B + (tx + 8 * j) * BS_LD + 8 * kq);
+        const ulonglong2 b1 = *reinterpret_cast<const ulonglong2 *>(B + (tx + 8 * j) * BS_LD + 8 * kq + 4);
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          b[j][0] = *reinterpret_cast<const float4 *>(&st.B[m][tx + 16 * j][8 * kq]);
-          b[j][1] = *reinterpret_cast<const float4 *>(&st.B[m][tx + 16 * j][8 * kq + 4]);
+        for (int r = 0; r < 8; ++r) {
+          acc[r][j] = fma2(a[r].x, b0.x, acc[r][j]);
+          acc[r][j] = fma2(a[r].y, b0.y, acc[r][j]);
+          acc[r][j] = fma2(a[r].z, b1.x, acc[r][j]);
+          acc[r][j] = fma2(a[r].w, b1.y, acc[r][j]);
         }
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            // b[j][0] = (re_k, im_k, re_k+1, im_k+1), b[j][1] the same for k+2, k+3
-            float sr = acc[m][r][j][0], si = acc[m][r][j][1];
-            sr = fmaf(a[r].x, b[j][0].x, sr);
-            si = fmaf(a[r].x, b[j][0].y, si);
-            sr = fmaf(a[r].y, b[j][0].z, sr);
-            si = fmaf(a[r].y, b[j][0].w, si);
-            sr = fmaf(a[r].z, b[j][1].x, sr);
-            si = fmaf(a[r].z, b[j][1].y, si);
-            sr = fmaf(a[r].w, b[j][1].z, sr);
-            si = fmaf(a[r].w, b[j][1].w, si);
-            acc[m][r][j][0] = sr;
-            acc[m][r][j][1] = si;
-          }
       }
     }
-    __syncthreads();
+    named_bar_sync(1 + m, GT);
   }
 
   const float thr = tile_threshold(P);
   const bool store = (P.lnl_tile != nullptr);
   const float zs = P.z_scale / (P.g_scale ? *P.g_scale : 1.f);
-  // epilogue: 4 rows x 2 extrinsic samples per thread, each thread's Z through its own
-  // column of shared memory (free after the mainloop), so that the pairs are a rolled loop
-  // and the accumulators' registers serve the evaluation
-  auto &zst = S.u.r.z;
+  __syncthreads();  // every mode's operands consumed: the stages become Z
 #pragma unroll
-  for (int k = 0; k < MAXM; ++k) {
-    const int mk = P.kmode[k];  // (zero where the bank has no such mode)
+  for (int r = 0; r < 8; ++r)
 #pragma unroll
-    for (int q = 0; q < 8; ++q)
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        float v = 0.f;
-#pragma unroll
-        for (int m = 0; m < MAXM; ++m) v = (m == mk) ? acc[m][q >> 1][q & 1][c] * zs : v;
-        zst[q][2 * k + c][tid] = v;
-      }
-  }
-  const bool pol = (P.n_pol == 2);
+    for (int j = 0; j < 4; ++j) {
+      stage[z_at(2 * m, ty + 8 * r, tx + 8 * j)] = __uint_as_float((uint32_t)acc[r][j]) * zs;
+      stage[z_at(2 * m + 1, ty + 8 * r, tx + 8 * j)] = __uint_as_float((uint32_t)(acc[r][j] >> 32)) * zs;
+    }
+  __syncthreads();
+
+  // a warp per row, a lane per sample
+  const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+  const bool pol = (P.n_pol == 2), ve = e0 + lane < P.n_ext;
+  const double lwe = S.lwe[lane];
+  Lse col, t1, t2;
+  col.init();
+  t1.init();
+  t2.init();
+  float best = -1.f;
+  long long barg = 0x7fffffffffffffffLL;
+  int np = 0;
 #pragma unroll 1
-  for (int q = 0; q < 8; ++q) {
-    const int rl = ty * 4 + (q >> 1), el = tx + 16 * (q & 1);
-    const int64_t i = i0 + rl, e = e0 + el;
-    float x = -INFINITY, x2 = -INFINITY, ml = -1.f;
-    int pk = 0;
-    if (i < P.n_int && e < P.n_ext) {
-      // the row's records are read through the cache for each pair
-      const float *mrow = P.mx + i * P.n_det * (pol ? REC_P : REC);
-      const double lwi = P.lw_int ? P.lw_int[i] : 0.0;
+  for (int rl = warp; rl < TI; rl += nw) {
+    const int64_t i = i0 + rl, e = e0 + lane;
+    if (i >= P.n_int) break;
+    float x = -INFINITY;
+    if (ve) {
       float Zr[MAXM], Zi[MAXM];
 #pragma unroll
       for (int k = 0; k < MAXM; ++k) {
-        Zr[k] = zst[q][2 * k][tid];
-        Zi[k] = zst[q][2 * k + 1][tid];
+        const int mk = P.kmode[k];  // (zero where the bank has no such mode)
+        Zr[k] = mk >= 0 ? stage[z_at(2 * mk, rl, lane)] : 0.f;
+        Zi[k] = mk >= 0 ? stage[z_at(2 * mk + 1, rl, lane)] : 0.f;
       }
       if (P.gemm_only) {
-        float sx = 0.f;
+        x = 0.f;
 #pragma unroll
-        for (int k = 0; k < MAXM; ++k) sx += Zr[k] + Zi[k];
-        x = sx; x2 = sx; ml = 0.f;
+        for (int k = 0; k < MAXM; ++k) x += Zr[k] + Zi[k];
+        t2.add(x);
+        best = fmaxf(best, 0.f);
       } else {
+        const float *mrow = P.mx + i * P.n_det * (pol ? REC_P : REC);
         float C0, Cr[3], Ci[3];
-        if (pol) hh_coeffs_pol(mrow, &qs[el * MAXD * REC], P, C0, Cr, Ci);
-        else hh_coeffs_by<false>([&](int k) { return __ldg(mrow + k); }, &qs[el * MAXD * REC], P, C0, Cr, Ci);
-        PairRes pr = pair_eval(Zr, Zi, C0, Cr, Ci, thr, !store, P, ph);
-        float lw = (float)(lwi + lwe[el]);
+        if (pol) hh_coeffs_pol(mrow, &S.qs[lane * QS_LD], P, C0, Cr, Ci);
+        else if (P.consec) hh_coeffs_by<true>([&](int k) { return __ldg(mrow + k); }, &S.qs[lane * QS_LD], P, C0, Cr, Ci);
+        else hh_coeffs_by<false>([&](int k) { return __ldg(mrow + k); }, &S.qs[lane * QS_LD], P, C0, Cr, Ci);
+        const PairRes pr = pair_eval(Zr, Zi, C0, Cr, Ci, thr, !store, P, S.ph);
+        const float lw = (float)((P.lw_int ? P.lw_int[i] : 0.0) + lwe);
         x = pr.lsum + lw;
-        x2 = pr.lsum2 + 2.f * lw;
-        ml = pr.ml;
-        pk = pr.argo | (pr.npass << 16);
+        t2.add(pr.lsum2 + 2.f * lw);
+        np += pr.npass;
+        const long long gi = (i * P.n_ext + e) * (long long)P.n_phi + pr.argo;
+        if (pr.ml > best || (pr.ml == best && gi < barg)) { best = pr.ml; barg = gi; }
         if (store) {
           P.lnl_tile[i * P.n_ext + e] = pr.lsum - P.ln_nphi;
           P.ml_tile[i * P.n_ext + e] = pr.ml;
         }
       }
     }
-    xs[rl][el] = x;
-    x2s[rl][el] = x2;
-    mls[rl][el] = ml;
-    pks[rl][el] = pk;
+    col.add(x);
+    Lse row;
+    row.init();
+    row.add(x);
+    warp_merge_lse(row);
+    t1.merge(row.m, row.s);
+    if (lane == 0) P.row_part[(int64_t)et * P.n_int + i] = make_float2(row.m, row.s);
+  }
+  S.col[warp][lane] = make_float2(col.m, col.s);
+  warp_merge_lse(t2);
+  warp_argmax(best, barg);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) np += __shfl_xor_sync(0xffffffffu, np, o);
+  if (lane == 0) {
+    S.w_m1[warp] = t1.m; S.w_s1[warp] = t1.s; S.w_m2[warp] = t2.m; S.w_s2[warp] = t2.s;
+    S.w_ml[warp] = best; S.w_arg[warp] = barg; S.w_np[warp] = np;
   }
   __syncthreads();
-
-  const int64_t tile = (int64_t)it * gridDim.x + et;
-  if (tid < TI) {
-    // row partials over the tile's extrinsic samples
-    Lse a, b;
-    a.init(); b.init();
-    float best = -1.f;
-    long long barg = 0;
-    int np = 0;
-    for (int c = 0; c < TE; ++c) {
-      a.add(xs[tid][c]);
-      b.add(x2s[tid][c]);
-      int pk = pks[tid][c];
-      np += pk >> 16;
-      float v = mls[tid][c];
-      if (v > best) { best = v; barg = ((i0 + tid) * P.n_ext + e0 + c) * (long long)P.n_phi + (pk & 0xFFFF); }
-    }
-    if (i0 + tid < P.n_int) P.row_part[(int64_t)et * P.n_int + i0 + tid] = make_float2(a.m, a.s);
-    r_m1[tid] = a.m; r_s1[tid] = a.s; r_m2[tid] = b.m; r_s2[tid] = b.s;
-    r_ml[tid] = best; r_arg[tid] = barg; r_np[tid] = np;
-  } else if (tid < TI + TE) {
-    const int c = tid - TI;
+  if (tid < TE) {
     Lse a;
     a.init();
-    for (int rr = 0; rr < TI; ++rr) a.add(xs[rr][c]);
-    if (e0 + c < P.n_ext) P.col_part[(int64_t)it * P.n_ext + e0 + c] = make_float2(a.m, a.s);
+    for (int q = 0; q < nw; ++q) a.merge(S.col[q][tid].x, S.col[q][tid].y);
+    if (e0 + tid < P.n_ext) P.col_part[(int64_t)it * P.n_ext + e0 + tid] = make_float2(a.m, a.s);
   }
-  __syncthreads();
-  if (tid < 32) {
+  if (tid == 32) {
     Lse a, b;
-    a.init(); b.init();
-    float best = -1.f;
-    long long barg = 0x7fffffffffffffffLL;
-    int np = 0;
-    for (int rr = tid; rr < TI; rr += 32) {
-      a.merge(r_m1[rr], r_s1[rr]);
-      b.merge(r_m2[rr], r_s2[rr]);
-      np += r_np[rr];
-      if (r_ml[rr] > best || (r_ml[rr] == best && r_arg[rr] < barg)) { best = r_ml[rr]; barg = r_arg[rr]; }
+    a.init();
+    b.init();
+    float bv = -1.f;
+    long long bi = 0x7fffffffffffffffLL;
+    int n = 0;
+    for (int q = 0; q < nw; ++q) {
+      a.merge(S.w_m1[q], S.w_s1[q]);
+      b.merge(S.w_m2[q], S.w_s2[q]);
+      n += S.w_np[q];
+      if (S.w_ml[q] > bv || (S.w_ml[q] == bv && S.w_arg[q] < bi)) { bv = S.w_ml[q]; bi = S.w_arg[q]; }
     }
-    warp_merge_lse(a);
-    warp_merge_lse(b);
-    warp_argmax(best, barg);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) np += __shfl_xor_sync(0xffffffffu, np, o);
-    if (tid == 0) {
-      P.tile_part[tile] = make_float4(a.m, a.s, b.m, b.s);
-      P.tile_ml[tile] = best;
-      P.tile_arg[tile] = barg;
-      P.tile_npass[tile] = np;
-      if (best > 0.f && P.track_max) atomic_max_nonneg(P.ml_running, best);
-    }
+    const int64_t tile = (int64_t)it * gridDim.x + et;
+    P.tile_part[tile] = make_float4(a.m, a.s, b.m, b.s);
+    P.tile_ml[tile] = bv;
+    P.tile_arg[tile] = bi;
+    P.tile_npass[tile] = n;
+    if (bv > 0.f && P.track_max) atomic_max_nonneg(P.ml_running, bv);
   }
 }
 
 void launch_simt(const SimtArgs &g, const EpiParams &P, cudaStream_t st) {
   dim3 grid((unsigned)((P.n_ext + TE - 1) / TE), (unsigned)((P.n_int + TI - 1) / TI));
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(simt_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SimtSmem));
-    attr = true;
-  }
-  simt_fused_kernel<<<grid, NT, sizeof(SimtSmem), st>>>(g, P);
+  cudaFuncSetAttribute(simt_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)(stage_bytes(MAXM) + sizeof(SimtSmem)));
+  simt_fused_kernel<<<grid, GT * P.n_modes, stage_bytes(P.n_modes) + sizeof(SimtSmem), st>>>(g, P);
 }
 
 }  // namespace dotpe
