@@ -1246,7 +1246,8 @@ static int preselect_locked(dotpe_ctx *ctx, const dotpe_presel_desc *d, float *l
   const bool bf = prec_bf16(prec), split = prec_split(prec);
   const int planes = split ? 2 : 1;
   const int J = M * (polb ? 2 : 1);  // data-weight components: (mode, polarisation) pairs j = 2m + p
-  const int MG = rb ? J : 1;          // time-grid operands: one per component with relative binning
+  // time-grid operands: one per component with relative binning (the FP32 kernel weights the rows instead)
+  const int MG = rb && !simt_pol ? J : 1;
   cudaStream_t st = ctx->main_stream;
 
   // cross-term records: the bank's cache entry for this PSD, a new one when the
@@ -1323,6 +1324,7 @@ static int preselect_locked(dotpe_ctx *ctx, const dotpe_presel_desc *d, float *l
   pa.G32 = (float2 *)(scr + o_G); pa.gmax = (float *)(scr + o_gmax);
   pa.gpack = scr + o_pack; pa.pack_kind = polb ? 0 : (bf ? 1 : 2); pa.pack_planes = planes;
   pa.gscale = (float *)(scr + o_gs); pa.status = status;
+  pa.unit = rb && simt_pol;
   launch_presel_prep(pa, st);
   if (simt_pol) launch_transpose_G((int64_t)MG * D, NTP, B, pa.G32, (float2 *)(scr + o_GT), st);
   if (polb && !simt_pol)
@@ -1427,7 +1429,7 @@ static int preselect_locked(dotpe_ctx *ctx, const dotpe_presel_desc *d, float *l
       for (int m = 0; m < MAXM; ++m) pp.mode_m[m] = m < M ? b.mode_m[m] : 0;
       pp.master = b.master;
       pp.G = (const float2 *)(scr + o_GT);
-      pp.n_gcomp = MG;
+      pp.c = rb ? pa.c : nullptr;
       pp.mx = mx;
       pp.rank_tol = PS_RANK_TOL;
       pp.keys = P.keys;

@@ -251,6 +251,7 @@ struct PreselPrepArgs {
   int pack_planes;       // 1 or 2 (hi, lo)
   float *gscale;         // 1 float out
   int *status;
+  int unit;              // one operand without data weights (the caller applies c itself)
 };
 void launch_presel_prep(const PreselPrepArgs &a, cudaStream_t st);
 struct PreselParams {
@@ -297,9 +298,10 @@ struct PreselPolArgs {
   int n_det, n_t, n_tpad, n_phi, n_modes, n_bins, kpad;
   int mode_m[MAXM];
   const float *master;       // FP32 master [M][bank_rows][kpad], rows [Re h+ | Im h+ | Re hx | Im hx | 0]
-  const float2 *G;           // [n_gcomp][n_det][n_bins][n_tpad] time-grid operand c_kjb e^{-2 pi i f_b t_kt},
-                             // times innermost so that a warp's threads (times) read consecutive words
-  int n_gcomp;               // 1 (one operand for every component), or 2 n_modes with relative binning (j = 2m + p)
+  const float2 *G;           // [n_det][n_bins][n_tpad] time-grid operand c_kb e^{-2 pi i f_b t_kt}, times
+                             // innermost so that a warp's threads read consecutive words
+  const float2 *c;           // relative binning: the components' data weights [n_det][2 n_modes][n_bins]
+                             // (j = 2m + p), G then without weights; else null
   const float *mx;           // [n_rows][n_det][REC_P] overlap records (slice-relative)
   float rank_tol;
   unsigned long long *keys;  // [n_rows][n_det] out, zeroed

@@ -729,7 +729,8 @@ void launch_prep(const PrepArgs &a, cudaStream_t st) {
 // Pre-selection operand (Sec. IV.D, App. B): G_k[b, t] = c_{kb} e^{-2 pi i f_b t_{kt}}
 // ---------------------------------------------------------------------------
 // One matrix for every mode (plain quadrature), or one per mode when the data
-// weights are per mode (relative binning): G[mg][(d, t)][b], mg < n_gmodes.
+// weights are per mode (relative binning): G[mg][(d, t)][b], mg < n_gmodes.  c null: the
+// time shifts alone, one matrix.
 __global__ void presel_G_kernel(int D, int B, int M, int n_gmodes, int n_t, int n_tpad, const float *__restrict__ fh,
                                 const float *__restrict__ fl, const double *__restrict__ t_grid,
                                 const float2 *__restrict__ c, float2 *__restrict__ G, float *__restrict__ gmax,
@@ -748,8 +749,11 @@ __global__ void presel_G_kernel(int D, int B, int M, int n_gmodes, int n_t, int 
       if (!isfinite(tv)) { atomicCAS(status, 0, DEV_E_NONFINITE); tv = 0.0; }
       const float th = (float)tv, tl = (float)(tv - (double)th);
       const float2 T = shift_factor(fh[b], fl[b], th, tl);
-      const float2 cc = c[((int64_t)d * M + mg) * B + b];
-      g = make_float2(T.x * cc.x - T.y * cc.y, T.x * cc.y + T.y * cc.x);
+      g = T;
+      if (c) {
+        const float2 cc = c[((int64_t)d * M + mg) * B + b];
+        g = make_float2(T.x * cc.x - T.y * cc.y, T.x * cc.y + T.y * cc.x);
+      }
     }
     G[k] = g;
     a = fmaxf(fabsf(g.x), fabsf(g.y));
@@ -763,9 +767,10 @@ void launch_presel_prep(const PreselPrepArgs &a, cudaStream_t st) {
   const int DB = a.D * a.B;
   prep_bins_kernel<<<nblk(DB > a.B ? DB : a.B, 256), 256, 0, st>>>(a.D, a.B, a.M, a.f, a.w, a.psd, a.data,
                                                                    a.rb_dh, a.c, a.omega, a.fh, a.fl, a.status);
-  const int mg = a.rb_dh ? a.M : 1;
+  const int mg = (a.rb_dh && !a.unit) ? a.M : 1;
   const int64_t n = (int64_t)mg * a.D * a.n_tpad * a.B;
-  presel_G_kernel<<<nblk(n, 256), 256, 0, st>>>(a.D, a.B, a.M, mg, a.n_t, a.n_tpad, a.fh, a.fl, a.t_grid, a.c,
+  presel_G_kernel<<<nblk(n, 256), 256, 0, st>>>(a.D, a.B, a.M, mg, a.n_t, a.n_tpad, a.fh, a.fl, a.t_grid,
+                                                a.unit ? nullptr : a.c,
                                                 a.G32, a.gmax, a.status);
   if (a.pack_kind == 0) return;  // the FP32 operand is used as it is
   const int64_t E = (int64_t)a.D * a.n_tpad;
