@@ -397,10 +397,11 @@ int dotpe_event_submit(dotpe_ctx *ctx, const dotpe_event_desc *desc, uint64_t *e
 
 /* Queues n events that share one bank and one precision as one batch: they are
  * admitted together (the sum of their footprints) and run as one launch
- * sequence on one slot: every event's preparation, then one persistent fused
- * tcgen05 launch per 64 events whose work items are the events' tiles one
- * event after the other (mixed precision: one screening launch, one selection
- * over the batch, one refinement launch), then every event's reduction.  The
+ * sequence on one slot: every event's preparation, then the kernels of each
+ * large event (96 or more tiles of 128 x 32 pairs per SM), then one persistent
+ * fused tcgen05 launch per 64 of the others whose work items are their tiles
+ * one event after the other (mixed precision: one screening launch, one
+ * selection over them, one refinement launch), then every event's reduction.  The
  * sequence is captured as a CUDA graph (unless DOTPE_CONFIG_NO_GRAPHS) whose
  * executable is kept per slot and updated in place for the next batch.  Each
  * event's results are those it gets when submitted alone (same tiles, same

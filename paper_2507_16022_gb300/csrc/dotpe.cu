@@ -915,6 +915,7 @@ static int autotune_band(dotpe_ctx *ctx, Event &e, EventRun &R, cudaStream_t st)
 // graphs on, the sequence is captured once per launch and replayed through a
 // per-slot executable graph updated in place when the topology repeats.
 // ---------------------------------------------------------------------------
+constexpr int OWN_LAUNCH_TILES = 96;  // 128 x 32-pair tiles per SM from which an event launches on its own
 static int run_batch(dotpe_ctx *ctx, const std::vector<Event *> &evs, int slot) {
   NvtxRange nv("dotpe:batch");
   cudaStream_t st = ctx->streams[slot];
@@ -927,6 +928,20 @@ static int run_batch(dotpe_ctx *ctx, const std::vector<Event *> &evs, int slot) 
   }
   const int prec = evs[0]->prec;
   const bool mixed = (prec == DOTPE_PREC_MIXED);
+  // Large events launch their own kernels, in turn; the others share one launch.  An own
+  // launch reads the event's parameters from constant memory instead of shared memory and
+  // takes CTA pairs: about 5 us less per tile and SM (12 events of 121 to 414 tiles per SM:
+  // 86.8 ms in shared launches, 69.8 ms in their own), but its launches cost the host about
+  // 0.2 ms per event (events of 22 to 72 tiles per SM: 19.0 against 19.6 ms, of 6 to 18: 8.3
+  // against 10.4 ms).
+  std::vector<int> own, shared;
+  std::string form;  // which is which, for the key of the executable graph
+  for (int k = 0; k < n; ++k) {
+    const int64_t tiles = (evs[k]->NI + TC_TI - 1) / TC_TI * R[k].L.n_etile;
+    const bool o = prec == DOTPE_PREC_FP32 || tiles >= (int64_t)OWN_LAUNCH_TILES * ctx->n_sms;
+    (o ? own : shared).push_back(k);
+    form += o ? '1' : '0';
+  }
   int total_tiles = 0;
   for (int k = 0; k < n; ++k) total_tiles += (int)((evs[k]->NI + TC_TI - 1) / TC_TI) * R[k].L.n_etile;
   // batch-wide (event, tile) list of the refinement
@@ -955,18 +970,19 @@ static int run_batch(dotpe_ctx *ctx, const std::vector<Event *> &evs, int slot) 
       event_block(ctx, *evs[k], R[k], 0, evs[k]->NI, st);
       CUDA_OR_FAIL(record(evs[k]->ev_k0, st));
     }
-    if (prec == DOTPE_PREC_FP32) {
-      for (int k = 0; k < n; ++k) {
-        int r = event_fused(ctx, *evs[k], R[k], true, st);
-        if (r != DOTPE_OK) return r;
-      }
-    } else {
-      std::vector<TcWork> W(n);
-      for (int k0 = 0; k0 < n; k0 += TC_MAXB) {
-        const int m = std::min(TC_MAXB, n - k0);
+    for (int k : own) {
+      int r = event_fused(ctx, *evs[k], R[k], true, st);
+      if (r != DOTPE_OK) return r;
+    }
+    const int ns = (int)shared.size();
+    if (ns > 0) {
+      std::vector<TcWork> W(ns);
+      for (int k0 = 0; k0 < ns; k0 += TC_MAXB) {
+        const int m = std::min(TC_MAXB, ns - k0);
         for (int k = k0; k < k0 + m; ++k) {
-          W[k] = R[k].W;
-          W[k].P = mixed ? screen_params(R[k]) : R[k].P;
+          EventRun &Rk = R[shared[k]];
+          W[k] = Rk.W;
+          W[k].P = mixed ? screen_params(Rk) : Rk.P;
         }
         TcLaunch T1 = T;
         T1.split = prec_split(prec) && !mixed;
@@ -974,28 +990,29 @@ static int run_batch(dotpe_ctx *ctx, const std::vector<Event *> &evs, int slot) 
         // one tile width for the launch: 64 samples only if every event takes it
         T1.tev = 64;
         for (int k = k0; k < k0 + m; ++k)
-          T1.tev = std::min(T1.tev, launch_tev(ctx, *evs[k], R[k].L, W[k].P, T1.split));
+          T1.tev = std::min(T1.tev, launch_tev(ctx, *evs[shared[k]], R[shared[k]].L, W[k].P, T1.split));
         if (mixed && T1.tev == 64)
           for (int k = k0; k < k0 + m; ++k) {
-            int rb = hh_bound_pass(ctx, *evs[k], R[k], W[k].P, st);
+            int rb = hh_bound_pass(ctx, *evs[shared[k]], R[shared[k]], W[k].P, st);
             if (rb != DOTPE_OK) return rb;
           }
         int r = launch_tc(T1, &W[k0], m, nullptr, nullptr, st);
         if (r != 0) return fail(DOTPE_E_DEVICE, "tcgen05 batch launch failed: %s", cudaGetErrorString((cudaError_t)r));
       }
       if (mixed) {
-        for (int k = 0; k < n; ++k) CUDA_OR_FAIL(record(evs[k]->ev_ks, st));
+        for (int k : shared) CUDA_OR_FAIL(record(evs[k]->ev_ks, st));
         int2 *glist = (int2 *)(blist + o_list);
         int *gn = (int *)(blist + o_n);
-        for (int k0 = 0; k0 < n; k0 += TC_MAXB) {
-          const int m = std::min(TC_MAXB, n - k0);
+        for (int k0 = 0; k0 < ns; k0 += TC_MAXB) {
+          const int m = std::min(TC_MAXB, ns - k0);
           SelectBatch sb;
           memset(&sb, 0, sizeof(sb));
           int b0 = 0;
           for (int k = 0; k < m; ++k) {
-            sb.ev[k] = select_event_of(R[k0 + k]);
+            const EventRun &Rk = R[shared[k0 + k]];
+            sb.ev[k] = select_event_of(Rk);
             sb.begin[k] = b0;
-            b0 += R[k0 + k].W.n_itile * R[k0 + k].W.n_etile;
+            b0 += Rk.W.n_itile * Rk.W.n_etile;
           }
           sb.begin[m] = b0;
           sb.n = m;
@@ -1005,7 +1022,7 @@ static int run_batch(dotpe_ctx *ctx, const std::vector<Event *> &evs, int slot) 
           sb.sep = (int *)(blist + o_sep);
           launch_select(sb, st);
           CUDA_OR_FAIL(cudaGetLastError());
-          for (int k = k0; k < k0 + m; ++k) W[k].P = refine_params(R[k]);
+          for (int k = k0; k < k0 + m; ++k) W[k].P = refine_params(R[shared[k]]);
           TcLaunch T2 = T;
           T2.split = true;
           T2.gate = sb.sep;
@@ -1037,8 +1054,7 @@ static int run_batch(dotpe_ctx *ctx, const std::vector<Event *> &evs, int slot) 
       return rc;
     }
     if (ce != cudaSuccess) return fail(DOTPE_E_DEVICE, "graph capture: %s", cudaGetErrorString(ce));
-    char key[64];
-    snprintf(key, sizeof(key), "%d/%d", n, prec);
+    const std::string key = form + "/" + std::to_string(prec);
     auto &cache = ctx->graphs[slot];
     auto it = cache.find(key);
     bool ok = false;
