@@ -143,14 +143,14 @@ struct Event {
   void *in_stage = nullptr;  // pinned host staging of host inputs
   size_t stage_bytes = 0;
   cudaEvent_t ev_inputs = nullptr, ev_start = nullptr, ev_end = nullptr, ev_k0 = nullptr, ev_k1 = nullptr,
-              ev_ks = nullptr;
+              ev_ks = nullptr;  // the kit's
   // results kept until release
   void *keep_block = nullptr;
   size_t keep_bytes = 0;
   double *ln_p_int = nullptr, *ln_p_ext = nullptr;
   float *lnl_tile = nullptr, *ml_tile = nullptr;
   ReduceOut *d_out = nullptr;
-  ReduceOut *h_out = nullptr;  // pinned
+  ReduceOut *h_out = nullptr;  // pinned, the kit's
   size_t scratch_bytes = 0;
   bool want_hb = false;  // admitted with room for the tensor-core <h|h> bound of its screen
   int slot = -1;
@@ -159,6 +159,24 @@ struct Event {
   float device_ms = -1.f, prep_ms = -1.f, fused_ms = -1.f, refine_ms = -1.f;
   int refined = -1;  // tiles refined (mixed precision)
 };
+
+// What every event needs and costs most to make: its CUDA events and the pinned result
+// record.  Released events give theirs back to the context (creating and destroying them and
+// the pinned staging took about 0.3 ms of a submit and release).
+struct EventKit {
+  cudaEvent_t inputs = nullptr, start = nullptr, end = nullptr, k0 = nullptr, k1 = nullptr, ks = nullptr;
+  ReduceOut *h_out = nullptr;  // pinned
+};
+struct Staging {
+  void *p;
+  size_t n;
+};
+constexpr size_t KITS_MAX = 64;                      // kept per context
+constexpr size_t STAGES_MAX = 8;                     // staging buffers kept per context, and
+constexpr size_t STAGES_BYTES = (size_t)64 << 20;    // their total size
+// Until the device writes an event's result: a completed record of a reused CUDA event is
+// not taken for this event's.
+constexpr int STATUS_PENDING = -0x7fffffff;
 
 }  // namespace dotpe
 
@@ -192,9 +210,78 @@ struct dotpe_ctx {
   std::unordered_map<uint64_t, int64_t> done_ns;
   bool stop = false;
   std::thread worker;
+  // spare parts of released events (under mu)
+  std::vector<dotpe::EventKit> kits;
+  std::vector<dotpe::Staging> stages;
+  size_t stages_bytes = 0;
 };
 
 namespace dotpe {
+
+static void kit_destroy(EventKit &k) {
+  for (cudaEvent_t e : {k.inputs, k.start, k.end, k.k0, k.k1, k.ks})
+    if (e) cudaEventDestroy(e);
+  if (k.h_out) cudaFreeHost(k.h_out);
+  k = EventKit();
+}
+
+static cudaError_t kit_take(dotpe_ctx *ctx, EventKit &k) {
+  if (!ctx->kits.empty()) {
+    k = ctx->kits.back();
+    ctx->kits.pop_back();
+    return cudaSuccess;
+  }
+  cudaError_t e = cudaEventCreateWithFlags(&k.inputs, cudaEventDisableTiming);
+  for (cudaEvent_t *v : {&k.start, &k.end, &k.k0, &k.k1, &k.ks})
+    if (e == cudaSuccess) e = cudaEventCreate(v);
+  if (e == cudaSuccess) e = cudaHostAlloc((void **)&k.h_out, sizeof(ReduceOut), cudaHostAllocDefault);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    kit_destroy(k);
+  }
+  return e;
+}
+
+static void kit_give(dotpe_ctx *ctx, EventKit &k) {
+  if (!k.h_out) return;
+  if (ctx->kits.size() < KITS_MAX) ctx->kits.push_back(k);
+  else kit_destroy(k);
+  k = EventKit();
+}
+
+// Pinned staging of at least n bytes: the smallest spare one that is not many times too
+// large, or a new one.
+static cudaError_t stage_take(dotpe_ctx *ctx, size_t n, void **p, size_t *size) {
+  size_t best = ctx->stages.size();
+  for (size_t q = 0; q < ctx->stages.size(); ++q)
+    if (ctx->stages[q].n >= n && ctx->stages[q].n <= std::max<size_t>(4 * n, (size_t)1 << 20) &&
+        (best == ctx->stages.size() || ctx->stages[q].n < ctx->stages[best].n))
+      best = q;
+  if (best < ctx->stages.size()) {
+    *p = ctx->stages[best].p;
+    *size = ctx->stages[best].n;
+    ctx->stages_bytes -= *size;
+    ctx->stages.erase(ctx->stages.begin() + best);
+    return cudaSuccess;
+  }
+  *size = (n + 65535) / 65536 * 65536;
+  const cudaError_t e = cudaHostAlloc(p, *size, cudaHostAllocDefault);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    *p = nullptr;
+  }
+  return e;
+}
+
+static void stage_give(dotpe_ctx *ctx, void *p, size_t n) {
+  if (!p) return;
+  if (ctx->stages.size() < STAGES_MAX && ctx->stages_bytes + n <= STAGES_BYTES) {
+    ctx->stages.push_back({p, n});
+    ctx->stages_bytes += n;
+  } else {
+    cudaFreeHost(p);
+  }
+}
 
 struct DoneArg {
   dotpe_ctx *ctx;
@@ -755,7 +842,7 @@ static int xterms_acquire(dotpe_ctx *ctx, Event &e, EventRun &R, cudaStream_t st
   return DOTPE_OK;
 }
 
-// Cross-term cache key: FNV-1a over n_det and the PSD bytes (host or device),
+// Cross-term cache key: an FNV-1a-like hash, a word at a time, of n_det and the PSD (host or device),
 // or, with relative binning, over a tag, n_det and the <h|h> weights (complex
 // [D][M][M][B]: n = 2 D M M B doubles), which then replace the PSD.
 static int psd_hash(int D, int B, const double *psd, uint64_t *out, const double *rb_hh = nullptr, size_t n_rb = 0) {
@@ -768,14 +855,20 @@ static int psd_hash(int D, int B, const double *psd, uint64_t *out, const double
   } else {
     memcpy(ps.data(), src, ps.size() * 8);
   }
+  // (the byte-wise form took 1.2 ms for the 1.2 MB of a polarisation-resolved bank's weights)
   uint64_t h = 1469598103934665603ull;
-  auto mix = [&](const void *p, size_t n) {
-    const uint8_t *c = (const uint8_t *)p;
-    for (size_t k = 0; k < n; ++k) h = (h ^ c[k]) * 1099511628211ull;
+  auto mix = [&](uint64_t v) {
+    h = (h ^ v) * 0x9e3779b97f4a7c15ull;
+    h ^= h >> 29;
   };
-  if (rb) mix("relative binning", 16);
-  mix(&D, sizeof(D));
-  mix(ps.data(), ps.size() * 8);
+  mix(rb ? 2 : 1);
+  mix((uint64_t)D);
+  mix((uint64_t)ps.size());
+  for (double x : ps) {
+    uint64_t v;
+    memcpy(&v, &x, 8);
+    mix(v);
+  }
   *out = h;
   return DOTPE_OK;
 }
@@ -1097,6 +1190,7 @@ static void progress(dotpe_ctx *ctx) {
     Event &e = *kv.second;
     if (e.state == DOTPE_STATE_RUNNING) {
       cudaError_t q = cudaEventQuery(e.ev_end);
+      if (q == cudaSuccess && *(volatile int *)&e.h_out->status == STATUS_PENDING) continue;
       if (q == cudaSuccess) {
         e.state = (e.h_out->status == 0) ? DOTPE_STATE_DONE : DOTPE_STATE_FAILED;
         {
@@ -1120,10 +1214,8 @@ static void progress(dotpe_ctx *ctx) {
         }
         ctx->used = (ctx->used >= e.scratch_bytes) ? ctx->used - e.scratch_bytes : 0;
         e.scratch_bytes = 0;
-        if (e.in_stage) {
-          cudaFreeHost(e.in_stage);
-          e.in_stage = nullptr;
-        }
+        stage_give(ctx, e.in_stage, e.stage_bytes);
+        e.in_stage = nullptr;
       } else if (q != cudaErrorNotReady) {
         cudaGetLastError();
         e.state = DOTPE_STATE_FAILED;
@@ -1197,6 +1289,7 @@ static void progress(dotpe_ctx *ctx) {
       for (Event *x : grp) {
         x->state = DOTPE_STATE_FAILED;
         x->launch_error = g_last_error;
+        if (x->h_out->status == STATUS_PENDING) x->h_out->status = 0;  // (no device status)
       }
       ctx->slot_busy[slot] = 0;
     }
@@ -1204,18 +1297,23 @@ static void progress(dotpe_ctx *ctx) {
 }
 
 static void free_event(dotpe_ctx *ctx, Event *e) {
-  if (e->state == DOTPE_STATE_RUNNING) cudaEventSynchronize(e->ev_end);
+  // Nothing of a finished event is in use any more.  Otherwise wait: a running event for its
+  // stream, one that failed part way for whatever it launched, a queued one for its inputs'
+  // copies (they read the staging buffer).
+  if (e->state != DOTPE_STATE_DONE) {
+    if (e->slot >= 0) cudaStreamSynchronize(ctx->streams[e->slot]);
+    if (e->ev_inputs) cudaEventSynchronize(e->ev_inputs);
+  }
   if (e->xent) e->xent->refs--;
-  if (e->keep_block) cudaFree(e->keep_block);
-  if (e->in_block && e->owns_inputs) cudaFree(e->in_block);
-  if (e->in_stage) cudaFreeHost(e->in_stage);
-  if (e->h_out) cudaFreeHost(e->h_out);
-  if (e->ev_inputs) cudaEventDestroy(e->ev_inputs);
-  if (e->ev_start) cudaEventDestroy(e->ev_start);
-  if (e->ev_end) cudaEventDestroy(e->ev_end);
-  if (e->ev_k0) cudaEventDestroy(e->ev_k0);
-  if (e->ev_k1) cudaEventDestroy(e->ev_k1);
-  if (e->ev_ks) cudaEventDestroy(e->ev_ks);
+  // (stream-ordered: a plain cudaFree would wait for the whole device)
+  if (e->keep_block) cudaFreeAsync(e->keep_block, ctx->input_stream);
+  if (e->in_block && e->owns_inputs) cudaFreeAsync(e->in_block, ctx->input_stream);
+  stage_give(ctx, e->in_stage, e->stage_bytes);
+  EventKit kit;
+  kit.inputs = e->ev_inputs; kit.start = e->ev_start; kit.end = e->ev_end;
+  kit.k0 = e->ev_k0; kit.k1 = e->ev_k1; kit.ks = e->ev_ks;
+  kit.h_out = e->h_out;
+  kit_give(ctx, kit);
   size_t give = e->keep_bytes + e->scratch_bytes + e->in_bytes;
   if (e->state == DOTPE_STATE_QUEUED) give = e->in_bytes;
   ctx->used = (ctx->used >= give) ? ctx->used - give : 0;
@@ -1773,6 +1871,8 @@ int dotpe_destroy(dotpe_ctx *ctx) {
     ctx->banks.clear();
   }
   cudaDeviceSynchronize();
+  for (auto &k : ctx->kits) kit_destroy(k);
+  for (auto &p : ctx->stages) cudaFreeHost(p.p);
   for (auto &m : ctx->graphs)
     for (auto &kv : m) cudaGraphExecDestroy(kv.second);
   for (auto s : ctx->streams) cudaStreamDestroy(s);
@@ -2279,8 +2379,9 @@ static int submit_locked(dotpe_ctx *ctx, const dotpe_event_desc *d, uint64_t gro
   // device copy of the inputs, ordered after the caller's stream
   cudaStream_t ist = ctx->input_stream;
   auto cleanup = [&](int rc) {
-    if (e->in_block) cudaFree(e->in_block);
-    if (e->in_stage) cudaFreeHost(e->in_stage);
+    cudaStreamSynchronize(ist);  // copies out of the staging buffer
+    if (e->in_block) cudaFreeAsync(e->in_block, ist);
+    stage_give(ctx, e->in_stage, e->stage_bytes);
     delete e;
     return rc;
   };
@@ -2313,11 +2414,8 @@ static int submit_locked(dotpe_ctx *ctx, const dotpe_event_desc *d, uint64_t gro
   for (auto &p : pieces)
     if (p.n && !is_device_ptr(p.src)) host_total += p.n;
   if (host_total) {
-    if (cudaHostAlloc(&e->in_stage, host_total, cudaHostAllocDefault) != cudaSuccess) {
-      cudaGetLastError();
+    if (stage_take(ctx, host_total, &e->in_stage, &e->stage_bytes) != cudaSuccess)
       return cleanup(fail(DOTPE_E_NOMEM, "pinned staging"));
-    }
-    e->stage_bytes = host_total;
   }
   if (d->stream) {
     cudaEvent_t dep;
@@ -2343,18 +2441,14 @@ static int submit_locked(dotpe_ctx *ctx, const dotpe_event_desc *d, uint64_t gro
                 : psd_hash(e->D, (int)B, d->psd, &e->psd_key);
     if (rc != DOTPE_OK) return cleanup(rc);
   }
-  cudaEventCreateWithFlags(&e->ev_inputs, cudaEventDisableTiming);
-  cudaEventCreate(&e->ev_start);
-  cudaEventCreate(&e->ev_end);
-  cudaEventCreate(&e->ev_k0);
-  cudaEventCreate(&e->ev_k1);
-  cudaEventCreate(&e->ev_ks);
+  EventKit kit;
+  if (kit_take(ctx, kit) != cudaSuccess) return cleanup(fail(DOTPE_E_NOMEM, "CUDA events or the pinned result"));
+  e->ev_inputs = kit.inputs; e->ev_start = kit.start; e->ev_end = kit.end;
+  e->ev_k0 = kit.k0; e->ev_k1 = kit.k1; e->ev_ks = kit.ks;
+  e->h_out = kit.h_out;
   cudaEventRecord(e->ev_inputs, ist);
-  if (cudaHostAlloc((void **)&e->h_out, sizeof(ReduceOut), cudaHostAllocDefault) != cudaSuccess) {
-    cudaGetLastError();
-    return cleanup(fail(DOTPE_E_NOMEM, "pinned result"));
-  }
   memset(e->h_out, 0, sizeof(ReduceOut));
+  e->h_out->status = STATUS_PENDING;
   e->id = ctx->next_id++;
   e->t_submit = now_ns();
   b->refs++;
@@ -2472,8 +2566,11 @@ int dotpe_event_wait(dotpe_ctx *ctx, uint64_t event_id, double timeout_s) {
                     it->second->launch_error.c_str());
       }
     }
-    if (timeout_s > 0 && (now_ns() - t0) > (int64_t)(timeout_s * 1e9)) return fail(DOTPE_E_TIMEOUT, "event wait");
-    std::this_thread::sleep_for(std::chrono::microseconds(20));
+    const int64_t waited = now_ns() - t0;
+    if (timeout_s > 0 && waited > (int64_t)(timeout_s * 1e9)) return fail(DOTPE_E_TIMEOUT, "event wait");
+    // the first milliseconds without sleeping (a 20 us sleep takes about 75): short events end in them
+    if (waited < 2000000) std::this_thread::yield();
+    else std::this_thread::sleep_for(std::chrono::microseconds(20));
   }
 }
 
@@ -2631,12 +2728,21 @@ int dotpe_lnl_blocks(dotpe_ctx *ctx, uint64_t event_id, int64_t i0, int64_t i1, 
     if (!(e.flags & DOTPE_FLAG_STORE_LNL)) return recompute_block(ctx, e, i0, i1, e0, e1, what, out, ld);
     const float *src = (what == DOTPE_LNL_MARG ? e.lnl_tile : e.ml_tile) + i0 * e.NE + e0;
     CUDA_OR_FAIL(cudaMemcpy2D(out, ld * 4, src, e.NE * 4, (e1 - e0) * 4, i1 - i0, cudaMemcpyDefault));
+    // (a copy within the device returns before it is done; a release may give src away)
+    CUDA_OR_FAIL(cudaStreamSynchronize(0));
     return DOTPE_OK;
   }
   if (what == DOTPE_ROW_MARGINAL || what == DOTPE_COL_MARGINAL) {
     const bool row = what == DOTPE_ROW_MARGINAL;
     int64_t a = row ? i0 : e0, z = row ? i1 : e1, n = row ? e.NI : e.NE;
     if (a < 0 || z > n || z <= a) return fail(DOTPE_E_INVALID, "marginal range");
+    if (is_device_ptr(out)) {
+      // on the default stream, as a copy would be
+      launch_to_float(z - a, (row ? e.ln_p_int : e.ln_p_ext) + a, out, 0);
+      CUDA_OR_FAIL(cudaGetLastError());
+      CUDA_OR_FAIL(cudaStreamSynchronize(0));
+      return DOTPE_OK;
+    }
     std::vector<double> tmp(z - a);
     CUDA_OR_FAIL(cudaMemcpy(tmp.data(), (row ? e.ln_p_int : e.ln_p_ext) + a, (z - a) * 8, cudaMemcpyDeviceToHost));
     std::vector<float> f(z - a);

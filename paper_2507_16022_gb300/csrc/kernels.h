@@ -68,6 +68,7 @@ void launch_master_to_planes(int64_t n, const float *master, const float *amax, 
 // on first use in the current CUDA context of `device` (which must be current);
 // later calls return the same address.  DOTPE_OK, or an error code with `msg`.
 int shared_dm_table(int device, cudaStream_t st, float4 **tab, char *msg, size_t msg_len);
+void launch_to_float(int64_t n, const double *in, float *out, cudaStream_t st);
 void launch_dist_marg_eval(int64_t n, const float *dh, const float *hh, float u_min, const float4 *tab, float *out,
                            cudaStream_t st);
 constexpr int64_t DM_NOALLOC_MAX = 1 << 20;  // evaluations per allocation-free call

@@ -944,6 +944,15 @@ int shared_dm_table(int device, cudaStream_t st, float4 **tab, char *msg, size_t
   return DOTPE_OK;
 }
 
+__global__ void to_float_kernel(int64_t n, const double *__restrict__ in, float *__restrict__ out) {
+  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (k < n) out[k] = (float)in[k];
+}
+
+void launch_to_float(int64_t n, const double *in, float *out, cudaStream_t st) {
+  to_float_kernel<<<nblk(n, 256), 256, 0, st>>>(n, in, out);
+}
+
 void launch_dist_marg_eval(int64_t n, const float *dh, const float *hh, float u_min, const float4 *tab, float *out,
                            cudaStream_t st) {
   dist_marg_eval_kernel<<<nblk(n, 256), 256, 0, st>>>(n, dh, hh, u_min, tab, out);
