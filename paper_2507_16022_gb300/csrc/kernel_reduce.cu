@@ -10,6 +10,8 @@
 // A slice processed as several bank blocks merges each block's (max, sum) pairs,
 // its column marginals and its best ln L^ML into FP64 accumulators in block
 // order; the final kernel turns them into the evidence.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -23,8 +25,7 @@ constexpr int NQ = 3;    // log-sum-exp inputs of a bank block: tile m1, tile m2
 
 // ln P over partials [nparts][n] (row or column marginal).  A block takes 32
 // consecutive entries (coalesced) and splits the parts over its 8 thread rows;
-// each thread keeps an online (max, sum) in FP64 and the rows merge in shared
-// memory.  With acc != nullptr the value is merged into the FP64 accumulator
+// each thread keeps an online (max, FP64 sum) and the rows merge in shared memory.  With acc != nullptr the value is merged into the FP64 accumulator
 // acc[k] = (m, s) (s = 0: empty) instead of written to out.
 constexpr int LX = 32, LY = 8;
 
@@ -34,14 +35,13 @@ __device__ __forceinline__ void lse_add(double &m, double &s, double x, double w
   if (x > m) { s = s * exp(m - x) + w; m = x; }
   else s += w * exp(x - m);
 }
-// The same for FP32 partials: FP32 maximum and exponentials (the partials carry
-// FP32 precision), FP64 sum.
-__device__ __forceinline__ void lse_add_f(float &m, double &s, float x, float w) {
-  if (!(w > 0.f)) return;
-  if (!(s > 0.0)) { m = x; s = w; return; }
-  if (x > m) { s = s * (double)__expf(m - x) + (double)w; m = x; }
-  else s += (double)w * (double)__expf(x - m);
-}
+// A thread takes LG parts at a time: all LG loads are in flight together, the
+// products w exp(x - max) of the group are formed in FP32 with their rounding
+// errors (FMA) and summed in two floats (Knuth's TwoSum, ~2^-46 of the group's sum),
+// and one FP64 operation adds the group.  An FP64 multiply, add and two conversions
+// per part bound the kernel by the FP64 pipe (2 per clock and SM) at a third of the
+// bandwidth; with a group of 8 it streams the partials (figures at launch_reduce_block).
+constexpr int LG = 8;
 
 __global__ void __launch_bounds__(LX * LY) reduce_lines_kernel(int64_t n, int nparts, const float2 *__restrict__ part,
                                                                double *__restrict__ out, double2 *__restrict__ acc,
@@ -51,9 +51,33 @@ __global__ void __launch_bounds__(LX * LY) reduce_lines_kernel(int64_t n, int np
   float mf = 0.f;
   double s = 0.0;
   if (k < n)
-    for (int p = threadIdx.y; p < nparts; p += LY) {
-      const float2 v = part[(int64_t)p * n + k];
-      lse_add_f(mf, s, v.x, v.y);
+    for (int p = threadIdx.y * LG; p < nparts; p += LY * LG) {
+      const float2 *src = part + (int64_t)p * n + k;
+      float2 v[LG];
+      float gm = -INFINITY;
+#pragma unroll
+      for (int j = 0; j < LG; ++j) v[j] = (p + j < nparts) ? src[j * n] : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int j = 0; j < LG; ++j) {
+        if (!(v[j].y > 0.f)) v[j] = make_float2(-INFINITY, 0.f);  // empty
+        gm = fmaxf(gm, v[j].x);
+      }
+      if (gm == -INFINITY) continue;
+      float hi = 0.f, lo = 0.f;
+#pragma unroll
+      for (int j = 0; j < LG; ++j) {
+        const float e = __expf(v[j].x - gm);
+        const float q = __fmul_rn(v[j].y, e);
+        const float r = fmaf(v[j].y, e, -q);
+        const float t = __fadd_rn(hi, q);
+        const float u = __fsub_rn(t, hi);
+        lo += __fadd_rn(__fsub_rn(hi, __fsub_rn(t, u)), __fsub_rn(q, u)) + r;
+        hi = t;
+      }
+      const double g = (double)hi + (double)lo;
+      if (!(s > 0.0)) { mf = gm; s = g; }
+      else if (gm > mf) { s = s * (double)__expf(mf - gm) + g; mf = gm; }
+      else s += g * (double)__expf(gm - mf);
     }
   double m = mf;
   sm[threadIdx.y][threadIdx.x] = m;
@@ -225,23 +249,40 @@ __global__ void reduce_block_merge_kernel(ReduceArgs a, int nb, const float *__r
     if (ob > best || (ob == best && oa < arg)) { best = ob; arg = oa; }
     np += __shfl_xor_sync(0xffffffffu, np, o);
   }
-  if (lane != 0) return;
-  EvAcc c = a.first ? EvAcc{0.0, 0.0, 0.0, 0.0, 0.0, 0.0, -1.f, 0x7fffffffffffffffLL, 0} : *a.acc;
-  double *dst[NQ][2] = {{&c.s1_m, &c.s1_s}, {&c.s2_m, &c.s2_s}, {&c.pi_m, &c.pi_s}};
-  for (int q = 0; q < NQ; ++q)
-    if (m[q] != -INFINITY) acc_merge(*dst[q][0], *dst[q][1], m[q], sm[q]);
-  if (best > c.best || (best == c.best && arg < c.arg)) { c.best = best; c.arg = arg; }
-  c.n_marg += np;
-  *a.acc = c;
+  // The sums are the same in every lane: lane q < NQ merges pair q, lane NQ the maximum and the count
+  double *dst = &a.acc->s1_m;  // the (max, sum) pairs lie one after the other
+#pragma unroll
+  for (int q = 1; q < NQ; ++q)
+    if (lane == q) { m[0] = m[q]; sm[0] = sm[q]; dst += 2 * q; }
+  if (lane < NQ) {
+    double am = 0.0, as = 0.0;
+    if (!a.first) { am = dst[0]; as = dst[1]; }
+    if (m[0] != -INFINITY) acc_merge(am, as, m[0], sm[0]);
+    dst[0] = am;
+    dst[1] = as;
+  } else if (lane == NQ) {
+    float cb = a.first ? -1.f : a.acc->best;
+    long long ca = a.first ? 0x7fffffffffffffffLL : a.acc->arg;
+    if (best > cb || (best == cb && arg < ca)) { cb = best; ca = arg; }
+    a.acc->best = cb;
+    a.acc->arg = ca;
+    a.acc->n_marg = (a.first ? 0 : a.acc->n_marg) + np;
+  }
 }
 
 // After the last block: column marginals, Sum_e P_e^2 (two passes) and the evidence.
-__global__ void __launch_bounds__(1024) reduce_final_kernel(ReduceArgs a) {
+// The marginals' FP64 logarithms and exponentials are bound by the FP64 pipe, so
+// they are spread over up to NB blocks, each leaving the maximum of its 2 ln P_e and
+// the sum against it; the last kernel merges those in a fixed order (figures at
+// launch_reduce_final).
+__global__ void __launch_bounds__(RB) reduce_ext_kernel(ReduceArgs a, float *__restrict__ bmax,
+                                                        double *__restrict__ bsum) {
   __shared__ float shf[32];
   __shared__ double shd[32];
-  const EvAcc c = *a.acc;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t k0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   float mc = -INFINITY;
-  for (int64_t k = threadIdx.x; k < a.n_ext; k += blockDim.x) {
+  for (int64_t k = k0; k < a.n_ext; k += stride) {
     const double2 v = a.acc_col[k];
     const double l = (v.y > 0.0) ? v.x + log(v.y) : -INFINITY;
     a.ln_p_ext[k] = l;
@@ -250,22 +291,53 @@ __global__ void __launch_bounds__(1024) reduce_final_kernel(ReduceArgs a) {
   mc = block_max(mc, shf);
   double sc = 0.0;
   if (mc != -INFINITY)
-    for (int64_t k = threadIdx.x; k < a.n_ext; k += blockDim.x) {
+    for (int64_t k = k0; k < a.n_ext; k += stride) {
       const double l = a.ln_p_ext[k];
       if (l != -INFINITY) sc += exp(2.0 * l - (double)mc);
     }
   sc = block_sum(sc, shd);
-  if (threadIdx.x != 0) return;
-  auto lnv = [](double m, double s) { return (s > 0.0) ? m + log(s) : -INFINITY; };
-  const double l1 = lnv(c.s1_m, c.s1_s), l2 = lnv(c.s2_m, c.s2_s), lpi = lnv(c.pi_m, c.pi_s);
-  const double lpe = (mc == -INFINITY || !(sc > 0.0)) ? -INFINITY : (double)mc + log(sc);
+  if (threadIdx.x == 0) { bmax[blockIdx.x] = mc; bsum[blockIdx.x] = sc; }
+}
+
+__global__ void reduce_final_kernel(ReduceArgs a, int nb, const float *__restrict__ bmax,
+                                    const double *__restrict__ bsum) {
+  // One warp.  FP64 logarithms and exponentials are chains of ~40 dependent operations:
+  // those of a step run in one lane each, side by side.
+  const EvAcc c = *a.acc;
+  const int lane = threadIdx.x;
+  float mc = -INFINITY;
+  for (int b = lane; b < nb; b += 32) mc = fmaxf(mc, bmax[b]);
+  for (int o = 16; o > 0; o >>= 1) mc = fmaxf(mc, __shfl_xor_sync(0xffffffffu, mc, o));
+  double sc = 0.0;
+  for (int b = lane; b < nb; b += 32)
+    if (bsum[b] > 0.0) sc += bsum[b] * exp((double)bmax[b] - (double)mc);
+  for (int o = 16; o > 0; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
+  double x = 1.0;  // the argument of lane's logarithm
+  if (lane == 0) x = c.s1_s;
+  if (lane == 1) x = c.s2_s;
+  if (lane == 2) x = c.pi_s;
+  if (lane == 3) x = sc;
+  if (lane == 4) x = (double)a.n_int_total;
+  if (lane == 5) x = (double)a.n_ext;
+  if (lane == 6) x = (double)a.n_phi;
+  const double lx = log(x);
+  auto lnv = [&](int l, double m, double s) {
+    const double v = __shfl_sync(0xffffffffu, lx, l);
+    return (s > 0.0) ? m + v : -INFINITY;
+  };
+  const double l1 = lnv(0, c.s1_m, c.s1_s), l2 = lnv(1, c.s2_m, c.s2_s), lpi = lnv(2, c.pi_m, c.pi_s);
+  const double lpe = lnv(3, mc, sc);
+  const double ln_i = lnv(4, 0.0, 1.0), ln_e = lnv(5, 0.0, 1.0), ln_o = lnv(6, 0.0, 1.0);
+  const double ex = exp(2.0 * l1 - (lane == 0 ? l2 : lane == 1 ? lpi : lpe));
+  const double n_eff_int = __shfl_sync(0xffffffffu, ex, 1), n_eff_ext = __shfl_sync(0xffffffffu, ex, 2);
+  if (lane != 0) return;
   ReduceOut o;
   o.ln_s1 = l1;
   o.ln_s2 = l2;
-  o.ln_z = l1 - log((double)a.n_int_total) - log((double)a.n_ext) - log((double)a.n_phi);
-  o.n_eff = (l1 == -INFINITY) ? 0.0 : exp(2.0 * l1 - l2);
-  o.n_eff_int = (l1 == -INFINITY) ? 0.0 : exp(2.0 * l1 - lpi);
-  o.n_eff_ext = (l1 == -INFINITY) ? 0.0 : exp(2.0 * l1 - lpe);
+  o.ln_z = l1 - ln_i - ln_e - ln_o;
+  o.n_eff = (l1 == -INFINITY) ? 0.0 : ex;
+  o.n_eff_int = (l1 == -INFINITY) ? 0.0 : n_eff_int;
+  o.n_eff_ext = (l1 == -INFINITY) ? 0.0 : n_eff_ext;
   o.max_ml = c.best;
   o.arg = c.arg;
   o.n_marg = c.n_marg;
@@ -281,24 +353,45 @@ size_t reduce_scratch_bytes() {
   return (size_t)NB * (NQ * sizeof(float) + NQ * sizeof(double) + sizeof(float) + 2 * sizeof(long long)) + 256;
 }
 
+namespace {
+struct BlockScratch {  // per-block results of the parallel passes, in ReduceArgs::scratch
+  float *bmax;
+  double *bsum;
+  float *bml;
+  long long *barg, *bnp;
+  explicit BlockScratch(void *scratch) {
+    uint8_t *w = (uint8_t *)scratch;
+    bmax = (float *)w;
+    bsum = (double *)(w + NB * NQ * sizeof(float));
+    bml = (float *)(bsum + NB * NQ);
+    barg = (long long *)(((uintptr_t)(bml + NB) + 7) & ~(uintptr_t)7);
+    bnp = barg + NB;
+  }
+};
+}  // namespace
+
+// The two line reductions stream 84 MB of partials for 65,536 rows x 4,096 samples: 34 us
+// (67 us with FP64 operations per part); 106 us (238 us) over four blocks of 65,536 rows
+// x 2,048 samples.
 void launch_reduce_block(const ReduceArgs &a, cudaStream_t st) {
   const dim3 lb(LX, LY);
   reduce_lines_kernel<<<(unsigned)((a.n_int + LX - 1) / LX), lb, 0, st>>>(a.n_int, a.n_etile, a.row_part,
                                                                          a.ln_p_int + a.row_offset, nullptr, 0);
   reduce_lines_kernel<<<(unsigned)((a.n_ext + LX - 1) / LX), lb, 0, st>>>(a.n_ext, a.n_itile, a.col_part, nullptr,
                                                                          a.acc_col, a.first);
-  uint8_t *w = (uint8_t *)a.scratch;
-  float *bmax = (float *)w;
-  double *bsum = (double *)(w + NB * NQ * sizeof(float));
-  float *bml = (float *)(bsum + NB * NQ);
-  long long *barg = (long long *)(((uintptr_t)(bml + NB) + 7) & ~(uintptr_t)7);
-  long long *bnp = barg + NB;
-  reduce_pass1_kernel<<<NB, RB, 0, st>>>(a, bmax, bml, barg, bnp);
-  reduce_pass2_kernel<<<NB, RB, 0, st>>>(a, bmax, bsum);
-  reduce_block_merge_kernel<<<1, 32, 0, st>>>(a, NB, bmax, bsum, bml, barg, bnp);
+  const BlockScratch s(a.scratch);
+  reduce_pass1_kernel<<<NB, RB, 0, st>>>(a, s.bmax, s.bml, s.barg, s.bnp);
+  reduce_pass2_kernel<<<NB, RB, 0, st>>>(a, s.bmax, s.bsum);
+  reduce_block_merge_kernel<<<1, 32, 0, st>>>(a, NB, s.bmax, s.bsum, s.bml, s.barg, s.bnp);
 }
 
-void launch_reduce_final(const ReduceArgs &a, cudaStream_t st) { reduce_final_kernel<<<1, 1024, 0, st>>>(a); }
+// 4,096 samples: 5.8 us for the marginals and 6.9 us for the record (24.8 us in one block).
+void launch_reduce_final(const ReduceArgs &a, cudaStream_t st) {
+  const int nb = (int)std::min<int64_t>(NB, (a.n_ext + RB - 1) / RB);
+  const BlockScratch s(a.scratch);
+  reduce_ext_kernel<<<nb, RB, 0, st>>>(a, s.bmax, s.bsum);
+  reduce_final_kernel<<<1, 32, 0, st>>>(a, nb, s.bmax, s.bsum);
+}
 
 // ---------------------------------------------------------------------------
 // Refinement selection (after a screening pass).  Tile t of event k is refined
