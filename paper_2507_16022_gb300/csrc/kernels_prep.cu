@@ -10,6 +10,9 @@
 //                             (Eq. hh_ieo)
 //  K2  cross_terms            row records <h_{im}|h_{im'}>_d = sum_b omega_{d,b} h h'^*
 //  K9  build_dm_table         FP64 Gauss-Legendre table of the distance-marginal remainder
+#include <cooperative_groups.h>
+
+#include <algorithm>
 #include <cstdio>
 #include <mutex>
 #include <type_traits>
@@ -19,6 +22,8 @@
 #include "kernels.h"
 
 namespace dotpe {
+
+namespace cg = cooperative_groups;
 
 // ---------------------------------------------------------------------------
 // K0
@@ -64,54 +69,82 @@ __global__ void prep_bins_kernel(int D, int B, int M, const double *__restrict__
   for (int m = 0; m < M; ++m) c[((int64_t)d * M + m) * B + b] = cv;
 }
 
+// The two norms below are sums of D B FP64 quotients.  One block took 12 us for them
+// (3 detectors x 512 bins; one SM divides at 2 FP64 operations per clock); a cluster of
+// NORM_CL blocks takes 6 us (rb_norm: 34 us before, 12 us now) and needs no buffer for the blocks' partial sums, which
+// rank 0 reads from their shared memory in rank order.
+constexpr int NORM_CL = 8, NORM_NT = 128;
+static_assert(2 * MAXM <= NORM_CL, "a block per component");
+
+// block sum (fixed order) in thread 0
+__device__ __forceinline__ double norm_block_sum(double v) {
+  __shared__ double part[NORM_NT / 32];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = 0.0;
+  for (int w = 0; w < NORM_NT / 32; ++w) v += part[w];
+  return v;
+}
+
 // Relative binning: the Cauchy-Schwarz scale of the screening margin,
 // sqrt(max_m sum_{d,b} |W^{<d|h>}_{d m b}|^2 / W^{<h|h>}_{d m m b}) (with plain
-// weights the same sum is <d|d>), in FP64, one block, fixed order.
-__global__ void rb_norm_kernel(int D, int M, int B, const double2 *__restrict__ rb_dh,
-                               const double2 *__restrict__ rb_hh, float *__restrict__ sqrt_dd) {
-  __shared__ double part[256];
-  double best = 0.0;
-  for (int m = 0; m < M; ++m) {
-    double v = 0.0;
-    for (int k = threadIdx.x; k < D * B; k += blockDim.x) {
+// weights the same sum is <d|d>), in FP64, one cluster, fixed order; the components
+// (M <= 2 MAXM = NORM_CL) share out the cluster's blocks.
+__global__ void __cluster_dims__(NORM_CL, 1, 1) __launch_bounds__(NORM_NT)
+rb_norm_kernel(int D, int M, int B, const double2 *__restrict__ rb_dh, const double2 *__restrict__ rb_hh,
+               float *__restrict__ sqrt_dd) {
+  __shared__ double sum;
+  cg::cluster_group cl = cg::this_cluster();
+  const int parts = NORM_CL / M, m = blockIdx.x / parts, p = blockIdx.x % parts;
+  double v = 0.0;
+  if (m < M)
+    for (int k = p * NORM_NT + threadIdx.x; k < D * B; k += parts * NORM_NT) {
       const int d = k / B, b = k % B;
       const double2 a = rb_dh[((int64_t)d * M + m) * B + b];
       const double h = rb_hh[(((int64_t)d * M + m) * M + m) * B + b].x;
       if (h > 0.0 && isfinite(h)) v += (a.x * a.x + a.y * a.y) / h;
     }
-    part[threadIdx.x] = v;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-      if ((int)threadIdx.x < o) part[threadIdx.x] += part[threadIdx.x + o];
-      __syncthreads();
+  v = norm_block_sum(v);
+  if (threadIdx.x == 0) sum = v;
+  cl.sync();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    double best = 0.0;
+    for (int q = 0; q < M; ++q) {
+      double s = 0.0;
+      for (int r = 0; r < parts; ++r) s += *cl.map_shared_rank(&sum, q * parts + r);
+      best = fmax(best, s);
     }
-    best = fmax(best, part[0]);
-    __syncthreads();
+    *sqrt_dd = (float)sqrt(best);
   }
-  if (threadIdx.x == 0) *sqrt_dd = (float)sqrt(best);
+  cl.sync();  // no block leaves before its sum is read
 }
 
-// sqrt<d|d> = sqrt(sum_{d,b} omega_{d,b} |d_d(f_b)|^2) in FP64, one block, fixed order.
-__global__ void data_norm_kernel(int D, int B, const double *__restrict__ w, const double *__restrict__ psd,
-                                 const double2 *__restrict__ data, float *__restrict__ sqrt_dd) {
-  __shared__ double part[256];
+// sqrt<d|d> = sqrt(sum_{d,b} omega_{d,b} |d_d(f_b)|^2) in FP64, one cluster, fixed order.
+__global__ void __cluster_dims__(NORM_CL, 1, 1) __launch_bounds__(NORM_NT)
+data_norm_kernel(int D, int B, const double *__restrict__ w, const double *__restrict__ psd,
+                 const double2 *__restrict__ data, float *__restrict__ sqrt_dd) {
+  __shared__ double sum;
+  cg::cluster_group cl = cg::this_cluster();
   double v = 0.0;
-  for (int k = threadIdx.x; k < D * B; k += blockDim.x) {
+  for (int k = blockIdx.x * NORM_NT + threadIdx.x; k < D * B; k += NORM_CL * NORM_NT) {
     const double S = psd[k];
     const double2 dk = data[k];
     if (S > 0.0 && isfinite(S) && isfinite(dk.x) && isfinite(dk.y)) v += 4.0 * w[k % B] / S * (dk.x * dk.x + dk.y * dk.y);
   }
-  part[threadIdx.x] = v;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) part[threadIdx.x] += part[threadIdx.x + o];
-    __syncthreads();
+  v = norm_block_sum(v);
+  if (threadIdx.x == 0) sum = v;
+  cl.sync();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    double s = 0.0;
+    for (int r = 0; r < NORM_CL; ++r) s += *cl.map_shared_rank(&sum, r);
+    *sqrt_dd = (float)sqrt(s);
   }
-  if (threadIdx.x == 0) *sqrt_dd = (float)sqrt(part[0]);
+  cl.sync();
 }
 
 // F non-null (polarisation-resolved bank): the column record is (F+^2, F+ Fx, Fx^2)
-// of the real antenna patterns F [E][D][2] and R is not read.
+// of the real antenna patterns F [E][D][2], Rf keeps (F+, Fx) at [e][d][0] and R is not read.
 __global__ void prep_ext_kernel(int64_t E, int D, int M, const double *__restrict__ t,
                                 const double2 *__restrict__ R, const double *__restrict__ F,
                                 float *__restrict__ th, float *__restrict__ tl,
@@ -126,6 +159,7 @@ __global__ void prep_ext_kernel(int64_t E, int D, int M, const double *__restric
   if (F) {
     double fp = F[2 * k], fx = F[2 * k + 1];
     if (!isfinite(fp) || !isfinite(fx)) { atomicCAS(status, 0, DEV_E_NONFINITE); fp = 0.0; fx = 0.0; }
+    Rf[k * M] = make_float2((float)fp, (float)fx);
     float *q = qx + k * REC;
     q[0] = (float)(fp * fp);
     q[1] = (float)(fp * fx);
@@ -171,81 +205,124 @@ __device__ __forceinline__ float2 shift_factor(float fh, float fl, float th, flo
   return make_float2(c, -s);
 }
 
-__global__ void build_G_kernel(int64_t E, int D, int M, int B, const float *__restrict__ fh,
-                               const float *__restrict__ fl, const float *__restrict__ th,
-                               const float *__restrict__ tl, const float2 *__restrict__ c,
-                               const float2 *__restrict__ Rf, float2 *__restrict__ G /*[M][E][B]*/,
-                               float *__restrict__ gmax) {
-  int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (k >= E * B) return;
-  int64_t e = k / B;
-  int b = (int)(k % B);
-  float2 g[MAXM];
+// build_G: a block takes GB_NT bins of GB_E samples.  A thread keeps one bin and its
+// samples' sums, so the data weights are read once for GB_E samples, the sample and bin
+// indices need no division, and the block leaves one atomic maximum: one per thread, all
+// to the same word, held it back (4096 samples x 512 bins x 3 detectors, 4 modes: 51 us
+// before, 32 us now; 67 MB written).  Grid: blocks of bins in y, of samples in x.
+constexpr int GB_NT = 128, GB_E = 4;
+
+// block maximum of a >= 0 into gmax
+__device__ __forceinline__ void block_gmax(float a, float *gmax) {
+  __shared__ int mx;
+  if (threadIdx.x == 0) mx = 0;
+  __syncthreads();
+  const int w = __reduce_max_sync(0xffffffffu, __float_as_int(a));
+  if ((threadIdx.x & 31) == 0) atomicMax(&mx, w);
+  __syncthreads();
+  if (threadIdx.x == 0) atomicMax(reinterpret_cast<int *>(gmax), mx);
+}
+
+template <int MM>
+__global__ void __launch_bounds__(GB_NT)
+build_G_kernel(int64_t E, int D, int B, const float *__restrict__ fh, const float *__restrict__ fl,
+               const float *__restrict__ th, const float *__restrict__ tl, const float2 *__restrict__ c,
+               const float2 *__restrict__ Rf, float2 *__restrict__ G /*[MM][E][B]*/, float *__restrict__ gmax) {
+  const int64_t e0 = (int64_t)blockIdx.x * GB_E;
+  const int ne = (int)(E - e0 < GB_E ? E - e0 : GB_E);
+  float a = 0.f;
+  for (int b = blockIdx.y * GB_NT + threadIdx.x; b < B; b += gridDim.y * GB_NT) {
+    float2 g[GB_E][MM];
 #pragma unroll
-  for (int m = 0; m < MAXM; ++m) g[m] = make_float2(0.f, 0.f);
-  float f_h = fh[b], f_l = fl[b];
-  for (int d = 0; d < D; ++d) {
-    float2 T = shift_factor(f_h, f_l, th[e * D + d], tl[e * D + d]);
+    for (int j = 0; j < GB_E; ++j)
 #pragma unroll
-    for (int m = 0; m < MAXM; ++m) {
-      if (m >= M) break;
-      const float2 cc = c[((int64_t)d * M + m) * B + b];
-      const float2 W = make_float2(T.x * cc.x - T.y * cc.y, T.x * cc.y + T.y * cc.x);
-      float2 r = Rf[(e * D + d) * M + m];
-      g[m].x += r.x * W.x - r.y * W.y;
-      g[m].y += r.x * W.y + r.y * W.x;
+      for (int m = 0; m < MM; ++m) g[j][m] = make_float2(0.f, 0.f);
+    const float f_h = fh[b], f_l = fl[b];
+    for (int d = 0; d < D; ++d) {
+      float2 cc[MM];
+#pragma unroll
+      for (int m = 0; m < MM; ++m) cc[m] = c[((int64_t)d * MM + m) * B + b];
+#pragma unroll
+      for (int j = 0; j < GB_E; ++j) {
+        const int64_t ed = (e0 + (j < ne ? j : 0)) * D + d;  // a ragged block repeats its first sample
+        const float2 T = shift_factor(f_h, f_l, th[ed], tl[ed]);
+#pragma unroll
+        for (int m = 0; m < MM; ++m) {
+          const float2 W = make_float2(T.x * cc[m].x - T.y * cc[m].y, T.x * cc[m].y + T.y * cc[m].x);
+          const float2 r = Rf[ed * MM + m];
+          g[j][m].x += r.x * W.x - r.y * W.y;
+          g[j][m].y += r.x * W.y + r.y * W.x;
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < GB_E; ++j) {
+      if (j >= ne) break;
+#pragma unroll
+      for (int m = 0; m < MM; ++m) {
+        G[((int64_t)m * E + e0 + j) * B + b] = g[j][m];
+        a = fmaxf(a, fmaxf(fabsf(g[j][m].x), fabsf(g[j][m].y)));
+      }
     }
   }
-  float a = 0.f;
-#pragma unroll
-  for (int m = 0; m < MAXM; ++m) {
-    if (m >= M) break;
-    G[((int64_t)m * E + e) * B + b] = g[m];
-    a = fmaxf(a, fmaxf(fabsf(g[m].x), fabsf(g[m].y)));
-  }
-  atomic_max_nonneg(gmax, a);
+  block_gmax(a, gmax);
 }
 
 // Polarisation-resolved bank: G_{m p}[b, e] = sum_d F_{e d p} e^{-2 pi i f_b t_{e d}} c_{d m p b},
-// G [M][2][E][B] (Eq. dh_ieo with the polarisation index; real antenna patterns); the data
-// weights c [D][M][2][B] are per component (the same for both with plain quadrature).
-__global__ void build_G_pol_kernel(int64_t E, int D, int M, int B, const float *__restrict__ fh,
-                                   const float *__restrict__ fl, const float *__restrict__ th,
-                                   const float *__restrict__ tl, const float2 *__restrict__ c,
-                                   const double *__restrict__ F, float2 *__restrict__ G,
-                                   float *__restrict__ gmax) {
-  int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (k >= E * B) return;
-  int64_t e = k / B;
-  int b = (int)(k % B);
-  float2 g[MAXM][2];
-#pragma unroll
-  for (int m = 0; m < MAXM; ++m) { g[m][0] = make_float2(0.f, 0.f); g[m][1] = make_float2(0.f, 0.f); }
-  float f_h = fh[b], f_l = fl[b];
-  for (int d = 0; d < D; ++d) {
-    const float2 T = shift_factor(f_h, f_l, th[e * D + d], tl[e * D + d]);
-    const float fp = (float)F[(e * D + d) * 2], fx = (float)F[(e * D + d) * 2 + 1];
-#pragma unroll
-    for (int m = 0; m < MAXM; ++m) {
-      if (m >= M) break;
-      const float2 c0 = c[((int64_t)(d * M + m) * 2) * B + b], c1 = c[((int64_t)(d * M + m) * 2 + 1) * B + b];
-      const float2 W0 = make_float2(T.x * c0.x - T.y * c0.y, T.x * c0.y + T.y * c0.x);
-      const float2 W1 = make_float2(T.x * c1.x - T.y * c1.y, T.x * c1.y + T.y * c1.x);
-      g[m][0].x += fp * W0.x; g[m][0].y += fp * W0.y;
-      g[m][1].x += fx * W1.x; g[m][1].y += fx * W1.y;
-    }
-  }
+// G [MM][2][E][B] (Eq. dh_ieo with the polarisation index; real antenna patterns); the data
+// weights c [D][MM][2][B] are per component (the same for both with plain quadrature).
+// Same blocks, GP_E samples at a time; a block walks the samples (its weights stay in the
+// first-level cache): 41 us for 4096 samples x 512 bins x 3 detectors, 4 modes, 64 us with a
+// block per GP_E samples, 57 us with a thread per (sample, bin), an atomic maximum each and
+// the antenna patterns converted from FP64 on every use.  The mode bank's kernel, with half
+// the weights to read, is the slower for it (40 against 32 us).
+constexpr int GP_E = 2;
+constexpr unsigned GP_BLOCKS = 10 * 152;  // blocks of samples and bins together, for the 152 SMs
+
+template <int MM>
+__global__ void __launch_bounds__(GB_NT)
+build_G_pol_kernel(int64_t E, int D, int B, const float *__restrict__ fh, const float *__restrict__ fl,
+                   const float *__restrict__ th, const float *__restrict__ tl, const float2 *__restrict__ c,
+                   const float2 *__restrict__ Rf /*(F+, Fx) at [e][d][0]*/, float2 *__restrict__ G, float *__restrict__ gmax) {
   float a = 0.f;
+  for (int64_t e0 = (int64_t)blockIdx.x * GP_E; e0 < E; e0 += (int64_t)gridDim.x * GP_E)
+  for (int b = blockIdx.y * GB_NT + threadIdx.x; b < B; b += gridDim.y * GB_NT) {
+    const int ne = (int)(E - e0 < GP_E ? E - e0 : GP_E);
+    float2 g[GP_E][MM * 2];
 #pragma unroll
-  for (int m = 0; m < MAXM; ++m) {
-    if (m >= M) break;
+    for (int j = 0; j < GP_E; ++j)
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      G[(((int64_t)m * 2 + q) * E + e) * B + b] = g[m][q];
-      a = fmaxf(a, fmaxf(fabsf(g[m][q].x), fabsf(g[m][q].y)));
+      for (int m = 0; m < MM * 2; ++m) g[j][m] = make_float2(0.f, 0.f);
+    const float f_h = fh[b], f_l = fl[b];
+    for (int d = 0; d < D; ++d) {
+      float2 cc[MM * 2];
+#pragma unroll
+      for (int m = 0; m < MM * 2; ++m) cc[m] = c[((int64_t)d * MM * 2 + m) * B + b];
+#pragma unroll
+      for (int j = 0; j < GP_E; ++j) {
+        const int64_t ed = (e0 + (j < ne ? j : 0)) * D + d;
+        const float2 T = shift_factor(f_h, f_l, th[ed], tl[ed]);
+        const float2 F = Rf[ed * MM];
+#pragma unroll
+        for (int m = 0; m < MM * 2; ++m) {
+          const float2 W = make_float2(T.x * cc[m].x - T.y * cc[m].y, T.x * cc[m].y + T.y * cc[m].x);
+          const float p = (m & 1) ? F.y : F.x;
+          g[j][m].x += p * W.x;
+          g[j][m].y += p * W.y;
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < GP_E; ++j) {
+      if (j >= ne) break;
+#pragma unroll
+      for (int m = 0; m < MM * 2; ++m) {
+        G[((int64_t)m * E + e0 + j) * B + b] = g[j][m];
+        a = fmaxf(a, fmaxf(fabsf(g[j][m].x), fabsf(g[j][m].y)));
+      }
     }
   }
-  atomic_max_nonneg(gmax, a);
+  block_gmax(a, gmax);
 }
 
 // fp16 operands are scaled to magnitudes up to 2^14 instead of 1: the five
@@ -260,67 +337,82 @@ __device__ __forceinline__ float pow2_scale(float maxabs) {
   return ldexpf(1.0f, -ex);
 }
 
-// Real-ified operand rows: (e, re) = [Gr | -Gi], (e, im) = [Gi | Gr], K padded with zeros
-// (the bank rows use the same column order: [Re h | Im h | 0]).
-// kind: 0 = fp32 plane, 1 = bf16 hi, 2 = fp16 hi; nplanes == 2 adds the lo plane
-// RN(v - hi) of the same type.  One thread per (m, e, c): for c < B it reads
-// G[m][e][c] once and writes the four entries that hold it (columns c and B + c
-// of both rows); for c < Kpad - 2B it zeroes column 2B + c of both rows.
+// two neighbouring 16-bit elements, and their lo parts a plane further on
 template <typename T>
-__device__ __forceinline__ void put(void *out, int64_t total, int64_t k, float v, int nplanes) {
-  if constexpr (sizeof(T) == 4) {
-    ((float *)out)[k] = v;
+__device__ __forceinline__ void put2(T *o, int64_t plane, float a, float b, int nplanes) {
+  if constexpr (std::is_same<T, __nv_bfloat16>::value) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    *(__nv_bfloat162 *)o = h;
+    if (nplanes == 2)
+      *(__nv_bfloat162 *)(o + plane) = __floats2bfloat162_rn(a - __bfloat162float(h.x), b - __bfloat162float(h.y));
   } else {
-    T hi;
-    float hf;
-    if constexpr (std::is_same<T, __nv_bfloat16>::value) { hi = __float2bfloat16_rn(v); hf = __bfloat162float(hi); }
-    else { hi = __float2half_rn(v); hf = __half2float(hi); }
-    ((T *)out)[k] = hi;
-    if (nplanes == 2) {
-      if constexpr (std::is_same<T, __nv_bfloat16>::value) ((T *)out)[total + k] = __float2bfloat16_rn(v - hf);
-      else ((T *)out)[total + k] = __float2half_rn(v - hf);
+    const __half2 h = __floats2half2_rn(a, b);
+    *(__half2 *)o = h;
+    if (nplanes == 2)
+      *(__half2 *)(o + plane) = __floats2half2_rn(a - __low2float(h), b - __high2float(h));
+  }
+}
+
+// Real-ified operand rows: (e, re) = [Gr | -Gi], (e, im) = [Gi | Gr], K padded with zeros
+// (the bank rows use the same column order: [Re h | Im h | 0]); NP polarisation blocks
+// along K (1, or 2 for a polarisation-resolved bank): row (m, e, re) =
+// [Gr_0 | -Gi_0 | Gr_1 | -Gi_1 | 0], (m, e, im) = [Gi_0 | Gr_0 | Gi_1 | Gr_1 | 0].
+// T: FP32 plane (the CUDA-core kernel's, which interleaves the two rows as
+// [me][Kpad][2]), bf16 or fp16 hi plane [2 me + part][Kpad]; nplanes == 2 adds the lo
+// plane RN(v - hi) of the same type.
+// One warp per (m, e), two neighbouring columns of both rows per lane: a store covers a
+// full line and the only index arithmetic is the segment of a column (a thread per bin,
+// with a 64-bit division and eight 2-byte stores, took 66 us for 4096 samples x 4 modes,
+// K = 1024, two planes; this 35 us).  The pack is bound by its 134 MB of stores.
+constexpr int PK_ROWS = 8;  // warps of a block
+constexpr int PK_BLOCKS = 16 * 152;  // two waves of the 152 SMs (8 blocks of 256 threads each)
+
+template <typename T>
+__global__ void __launch_bounds__(32 * PK_ROWS)
+pack_G_kernel(int64_t E, int M, int B, int Kpad, int NP, const float2 *__restrict__ G,
+              const float *__restrict__ gmax, int kind, int nplanes, void *__restrict__ out,
+              float *__restrict__ scale_out) {
+  const float sc = (kind == 0) ? 1.0f : pow2_scale(*gmax) * (kind == 2 ? FP16_OPERAND_SCALE : 1.0f);
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0 && scale_out) *scale_out = sc;
+  const int64_t me = (int64_t)blockIdx.x * PK_ROWS + threadIdx.y;
+  if (me >= E * M) return;
+  int64_t m = 0, e = me;
+  while (e >= E) { e -= E; ++m; }
+  const float2 *g0 = G + ((m * NP) * E + e) * B;  // polarisation q: + q E B
+  const int64_t total = (int64_t)M * 2 * E * Kpad;
+  for (int c = 64 * blockIdx.y + 2 * threadIdx.x; c < Kpad; c += 64 * gridDim.y) {
+    float re[2], im[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      int r = c + j;
+      const float2 *g = g0;
+      if (NP == 2 && r >= 2 * B) { r -= 2 * B; g += E * B; }
+      re[j] = im[j] = 0.f;
+      if (r < 2 * B) {
+        const bool second = r >= B;
+        const float2 v = g[second ? r - B : r];
+        re[j] = (second ? -v.y : v.x) * sc;
+        im[j] = (second ? v.x : v.y) * sc;
+      }
+    }
+    if constexpr (sizeof(T) == 4) {
+      *(float4 *)((float *)out + (me * Kpad + c) * 2) = make_float4(re[0], im[0], re[1], im[1]);
+    } else {
+      T *o = (T *)out + 2 * me * Kpad + c;
+      put2<T>(o, total, re[0], re[1], nplanes);
+      put2<T>(o + Kpad, total, im[0], im[1], nplanes);
     }
   }
 }
 
 template <typename T>
-__global__ void pack_G_kernel(int64_t E, int M, int B, int Kpad, int NP, const float2 *__restrict__ G,
-                              const float *__restrict__ gmax, int kind, int nplanes, void *__restrict__ out,
-                              float *__restrict__ scale_out) {
-  // NP polarisation blocks along K (1, or 2 for a polarisation-resolved bank):
-  // row (m, e, re) = [Gr_0 | -Gi_0 | Gr_1 | -Gi_1 | 0], (m, e, im) = [Gi_0 | Gr_0 | Gi_1 | Gr_1 | 0]
-  const int pad = Kpad - 2 * NP * B;
-  const int P = B > pad ? B : pad;  // threads per (m, e)
-  const int64_t total = (int64_t)M * 2 * E * Kpad;
-  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const float sc = (kind == 0) ? 1.0f : pow2_scale(*gmax) * (kind == 2 ? FP16_OPERAND_SCALE : 1.0f);
-  if (k == 0 && scale_out) *scale_out = sc;
-  if (k >= (int64_t)M * E * P) return;
-  const int c = (int)(k % P);
-  const int64_t me = k / P;  // m * E + e
-  const int64_t m = me / E, e = me - m * E;
-  // element (part, column) of sample me: the 16-bit planes keep the two rows
-  // [2 me][Kpad] and [2 me + 1][Kpad] (tensor-core B rows); the FP32 operand of
-  // the CUDA-core kernel interleaves them, [me][Kpad][2] = (re row, im row) per column
-  auto at = [&](int part, int64_t col) -> int64_t {
-    if constexpr (sizeof(T) == 4) return (me * Kpad + col) * 2 + part;
-    else return (2 * me + part) * Kpad + col;
-  };
-  if (c < B) {
-    for (int q = 0; q < NP; ++q) {
-      const float2 g = G[((m * NP + q) * E + e) * B + c];
-      const float gr = g.x * sc, gi = g.y * sc;
-      const int o = 2 * q * B;
-      put<T>(out, total, at(0, o + c), gr, nplanes);
-      put<T>(out, total, at(0, o + B + c), -gi, nplanes);
-      put<T>(out, total, at(1, o + c), gi, nplanes);
-      put<T>(out, total, at(1, o + B + c), gr, nplanes);
-    }
-  }
-  if (c < pad) {
-    put<T>(out, total, at(0, 2 * NP * B + c), 0.f, nplanes);
-    put<T>(out, total, at(1, 2 * NP * B + c), 0.f, nplanes);
-  }
+static void launch_pack(int64_t E, int M, int B, int Kpad, int NP, const float2 *G, const float *gmax, int kind,
+                        int nplanes, void *out, float *scale_out, cudaStream_t st) {
+  // few rows (a pre-selection's time grid, a small event): their columns over several blocks
+  const int64_t rows = (E * M + PK_ROWS - 1) / PK_ROWS;
+  const int cols = (int)std::max<int64_t>(1, std::min<int64_t>((Kpad + 63) / 64, PK_BLOCKS / rows));
+  pack_G_kernel<T><<<dim3((unsigned)rows, cols), dim3(32, PK_ROWS), 0, st>>>(
+      E, M, B, Kpad, NP, G, gmax, kind, nplanes, out, scale_out);
 }
 
 // ---------------------------------------------------------------------------
@@ -694,6 +786,15 @@ __global__ void dist_marg_eval_kernel(int64_t n, const float *__restrict__ dh, c
 // ---------------------------------------------------------------------------
 static inline unsigned nblk(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
+template <typename F>
+static void by_modes(int M, F f) {
+  if (M == 1) f(std::integral_constant<int, 1>());
+  else if (M == 2) f(std::integral_constant<int, 2>());
+  else if (M == 3) f(std::integral_constant<int, 3>());
+  else f(std::integral_constant<int, 4>());
+  static_assert(MAXM == 4, "a case per mode count");
+}
+
 void launch_prep(const PrepArgs &a, cudaStream_t st) {
   const bool pol = (a.n_pol == 2);
   const int NP = pol ? 2 : 1;
@@ -701,28 +802,29 @@ void launch_prep(const PrepArgs &a, cudaStream_t st) {
   prep_bins_kernel<<<nblk((int64_t)a.D * a.B, 256), 256, 0, st>>>(a.D, a.B, a.M * NP, a.f, a.w, a.psd, a.data,
                                                                 a.rb_dh, a.c, a.omega, a.fh, a.fl, a.status);
   if (a.sqrt_dd) {
-    if (a.rb_dh) rb_norm_kernel<<<1, 256, 0, st>>>(a.D, a.M * NP, a.B, a.rb_dh, a.rb_hh, a.sqrt_dd);
-    else data_norm_kernel<<<1, 256, 0, st>>>(a.D, a.B, a.w, a.psd, a.data, a.sqrt_dd);
+    if (a.rb_dh) rb_norm_kernel<<<NORM_CL, NORM_NT, 0, st>>>(a.D, a.M * NP, a.B, a.rb_dh, a.rb_hh, a.sqrt_dd);
+    else data_norm_kernel<<<NORM_CL, NORM_NT, 0, st>>>(a.D, a.B, a.w, a.psd, a.data, a.sqrt_dd);
   }
   prep_ext_kernel<<<nblk(a.E * a.D, 256), 256, 0, st>>>(a.E, a.D, a.M, a.t, a.R, pol ? a.F : nullptr, a.th, a.tl,
                                                         a.Rf, a.qx, a.status);
-  if (pol)
-    build_G_pol_kernel<<<nblk(a.E * a.B, 256), 256, 0, st>>>(a.E, a.D, a.M, a.B, a.fh, a.fl, a.th, a.tl, a.c, a.F,
-                                                             a.G32, a.gmax);
-  else
-    build_G_kernel<<<nblk(a.E * a.B, 256), 256, 0, st>>>(a.E, a.D, a.M, a.B, a.fh, a.fl, a.th, a.tl, a.c, a.Rf,
-                                                         a.G32, a.gmax);
-  const int pad = a.Kpad - 2 * NP * a.B;
-  const int64_t n = (int64_t)a.M * a.E * (a.B > pad ? a.B : pad);
+  by_modes(a.M, [&](auto mm) {
+    constexpr int MM = decltype(mm)::value;
+    const unsigned nb = std::min(nblk(a.B, GB_NT), 65535u);
+    if (pol) {
+      const unsigned blocks = std::min(nblk(a.E, GP_E), std::max(1u, GP_BLOCKS / nb));
+      build_G_pol_kernel<MM><<<dim3(blocks, nb), GB_NT, 0, st>>>(a.E, a.D, a.B, a.fh, a.fl, a.th, a.tl, a.c, a.Rf,
+                                                                a.G32, a.gmax);
+    } else {
+      build_G_kernel<MM><<<dim3(nblk(a.E, GB_E), nb), GB_NT, 0, st>>>(a.E, a.D, a.B, a.fh, a.fl, a.th, a.tl, a.c, a.Rf,
+                                                                     a.G32, a.gmax);
+    }
+  });
   if (a.pack_kind == 0)
-    pack_G_kernel<float><<<nblk(n, 256), 256, 0, st>>>(a.E, a.M, a.B, a.Kpad, NP, a.G32, a.gmax, 0, 1, a.gpack,
-                                                       a.gscale);
+    launch_pack<float>(a.E, a.M, a.B, a.Kpad, NP, a.G32, a.gmax, 0, 1, a.gpack, a.gscale, st);
   else if (a.pack_kind == 1)
-    pack_G_kernel<__nv_bfloat16><<<nblk(n, 256), 256, 0, st>>>(a.E, a.M, a.B, a.Kpad, NP, a.G32, a.gmax, 1,
-                                                               a.pack_planes, a.gpack, a.gscale);
+    launch_pack<__nv_bfloat16>(a.E, a.M, a.B, a.Kpad, NP, a.G32, a.gmax, 1, a.pack_planes, a.gpack, a.gscale, st);
   else
-    pack_G_kernel<__half><<<nblk(n, 256), 256, 0, st>>>(a.E, a.M, a.B, a.Kpad, NP, a.G32, a.gmax, 2, a.pack_planes,
-                                                        a.gpack, a.gscale);
+    launch_pack<__half>(a.E, a.M, a.B, a.Kpad, NP, a.G32, a.gmax, 2, a.pack_planes, a.gpack, a.gscale, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -774,14 +876,10 @@ void launch_presel_prep(const PreselPrepArgs &a, cudaStream_t st) {
                                                 a.G32, a.gmax, a.status);
   if (a.pack_kind == 0) return;  // the FP32 operand is used as it is
   const int64_t E = (int64_t)a.D * a.n_tpad;
-  const int pad = a.Kpad - 2 * a.B;
-  const int64_t np = mg * E * (a.B > pad ? a.B : pad);
   if (a.pack_kind == 1)
-    pack_G_kernel<__nv_bfloat16><<<nblk(np, 256), 256, 0, st>>>(E, mg, a.B, a.Kpad, 1, a.G32, a.gmax, 1, a.pack_planes,
-                                                                a.gpack, a.gscale);
+    launch_pack<__nv_bfloat16>(E, mg, a.B, a.Kpad, 1, a.G32, a.gmax, 1, a.pack_planes, a.gpack, a.gscale, st);
   else
-    pack_G_kernel<__half><<<nblk(np, 256), 256, 0, st>>>(E, mg, a.B, a.Kpad, 1, a.G32, a.gmax, 2, a.pack_planes,
-                                                         a.gpack, a.gscale);
+    launch_pack<__half>(E, mg, a.B, a.Kpad, 1, a.G32, a.gmax, 2, a.pack_planes, a.gpack, a.gscale, st);
 }
 
 // GT[mat][b][t] = G[mat][t][b]: one thread per output element, t fastest, so
@@ -818,13 +916,10 @@ void launch_presel_pol_pack(int64_t n_cols, int B, int Kpad, const float2 *G32, 
                             int kind, int planes, void *out, float *scale_out, cudaStream_t st) {
   presel_pol_spread_kernel<<<nblk(4 * n_cols * B, 256), 256, 0, st>>>(n_cols, B, G32, Gp);
   const int64_t E = 2 * n_cols;
-  const int pad = Kpad - 4 * B;
-  const int64_t n = E * (B > pad ? B : pad);
   if (kind == 1)
-    pack_G_kernel<__nv_bfloat16><<<nblk(n, 256), 256, 0, st>>>(E, 1, B, Kpad, 2, Gp, gmax, 1, planes, out,
-                                                               scale_out);
+    launch_pack<__nv_bfloat16>(E, 1, B, Kpad, 2, Gp, gmax, 1, planes, out, scale_out, st);
   else
-    pack_G_kernel<__half><<<nblk(n, 256), 256, 0, st>>>(E, 1, B, Kpad, 2, Gp, gmax, 2, planes, out, scale_out);
+    launch_pack<__half>(E, 1, B, Kpad, 2, Gp, gmax, 2, planes, out, scale_out, st);
 }
 
 void launch_cross_terms(int64_t n_rows, int64_t row0, int64_t I_bank, int M, int D, int B, int Kpad,
