@@ -287,7 +287,7 @@ struct PreselOut {
 // pol: a polarisation-resolved bank (time-grid operand from launch_presel_pol_pack, 32 columns per tile)
 int launch_presel(const CUtensorMap &mapG, const CUtensorMap &mapBank, const PreselParams &p, bool bf16, bool split,
                   bool per_mode, bool pol, int n_sms, cudaStream_t st);
-void launch_presel_finish(int64_t n, int D, int n_phi, double delta, const unsigned long long *keys, float *ml,
+void launch_presel_finish(int64_t n, int D, int n_phi, double delta, unsigned long long *keys, float *ml,
                           int *arg_ot, double *inco, unsigned long long *max_bits /*zeroed*/, int64_t *sel,
                           PreselOut *out, cudaStream_t st);
 
