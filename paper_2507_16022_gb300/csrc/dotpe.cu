@@ -1614,11 +1614,14 @@ static int rb_weights_locked(dotpe_ctx *ctx, const dotpe_rb_desc *d, double *w_d
     if (nodes[b] < 0 || nodes[b] >= N || (b > 0 && nodes[b] <= nodes[b - 1]))
       return fail(DOTPE_E_INVALID, "nodes must be strictly increasing indices into f_fine (node %d = %lld)", b,
                   (long long)nodes[b]);
+  const std::vector<int64_t> first = rb_parts(B, nodes.data());
+  const int64_t n_parts = first[B];
   cudaStream_t st = ctx->main_stream;
   Carver c;
   const size_t o_f = c.take<double>(N), o_df = c.take<double>(N), o_psd = c.take<double>((size_t)D * N);
   const size_t o_data = c.take<double2>((size_t)D * N), o_h0 = c.take<double2>((size_t)M * N);
-  const size_t o_t0 = c.take<double>(D), o_nodes = c.take<int64_t>(B);
+  const size_t o_t0 = c.take<double>(D), o_nodes = c.take<int64_t>(B), o_first = c.take<int64_t>(B + 1);
+  const size_t o_part = c.take<double>((size_t)D * n_parts * rb_part_doubles(M));
   const size_t o_wdh = c.take<double2>((size_t)D * M * B), o_whh = c.take<double2>((size_t)D * M * M * B);
   const size_t o_st = c.take<int>(1);
   uint8_t *scr = nullptr;
@@ -1639,10 +1642,12 @@ static int rb_weights_locked(dotpe_ctx *ctx, const dotpe_rb_desc *d, double *w_d
   ck(cudaMemcpyAsync(scr + o_h0, d->h0, (size_t)M * N * 16, cudaMemcpyDefault, st), "copying h0");
   if (d->t0) ck(cudaMemcpyAsync(scr + o_t0, d->t0, D * 8, cudaMemcpyDefault, st), "copying t0");
   ck(cudaMemcpyAsync(scr + o_nodes, nodes.data(), B * 8, cudaMemcpyHostToDevice, st), "copying nodes");
+  ck(cudaMemcpyAsync(scr + o_first, first.data(), (B + 1) * 8, cudaMemcpyHostToDevice, st), "copying nodes");
   if (rc == DOTPE_OK) {
     launch_rb_weights(D, M, N, (const double *)(scr + o_f), (const double *)(scr + o_df),
                       (const double *)(scr + o_psd), (const double2 *)(scr + o_data), (const double2 *)(scr + o_h0),
-                      (const double *)(scr + o_t0), B, (const int64_t *)(scr + o_nodes), (double2 *)(scr + o_wdh),
+                      (const double *)(scr + o_t0), B, n_parts, (const int64_t *)(scr + o_nodes),
+                      (const int64_t *)(scr + o_first), (double *)(scr + o_part), (double2 *)(scr + o_wdh),
                       (double2 *)(scr + o_whh), (int *)(scr + o_st), st);
     ck(cudaGetLastError(), "relative-binning weights kernel");
   }

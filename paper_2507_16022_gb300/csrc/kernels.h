@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "common.cuh"
 
 namespace dotpe {
@@ -318,9 +320,14 @@ void launch_presel_pol_pack(int64_t n_cols, int B, int Kpad, const float2 *G32, 
                             int kind, int planes, void *out, float *scale_out, cudaStream_t st);
 
 // Relative-binning weights (App. A): kernel_rb.cu.  w_dh [D][M][B], w_hh [D][M][M][B].
+// first [B + 1]: rb_parts(B, node) of the host's node indices, n_parts its last entry; part: scratch of
+// D n_parts rb_part_doubles(M) doubles
+std::vector<int64_t> rb_parts(int B, const int64_t *node);
+size_t rb_part_doubles(int M);
 void launch_rb_weights(int D, int M, int64_t N, const double *ff, const double *dff, const double *psd,
-                       const double2 *data, const double2 *h0, const double *t0, int B, const int64_t *node,
-                       double2 *w_dh, double2 *w_hh, int *status, cudaStream_t st);
+                       const double2 *data, const double2 *h0, const double *t0, int B, int64_t n_parts,
+                       const int64_t *node, const int64_t *first, double *part, double2 *w_dh, double2 *w_hh,
+                       int *status, cudaStream_t st);
 
 // Posterior samples of a finished event: kernel_sample.cu.
 struct SampleArgs {
