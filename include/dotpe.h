@@ -99,7 +99,7 @@ typedef struct dotpe_ctx dotpe_ctx;
  * CTA pairs) and L2 bands on the first event of each shape, keep the fastest */
 #define DOTPE_CONFIG_AUTOTUNE 0x1
 #define DOTPE_CONFIG_NO_GRAPHS 0x2 /* launch batches directly instead of as captured CUDA graphs */
-/* Screening and GEMM-only launches of mode banks use 128 x 32-sample tiles
+/* Screens, and GEMM-only launches of mode banks, use 128 x 32-sample tiles
  * (two TMEM accumulator sets) instead of the default 128 x 64-sample tiles (one
  * set of N = 128 per mode, twice the MMA work per operand byte).  Results are
  * the same either way; with DOTPE_CONFIG_AUTOTUNE the tuner times both. */

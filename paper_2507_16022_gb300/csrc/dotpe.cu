@@ -200,7 +200,7 @@ struct dotpe_ctx {
   std::unordered_map<std::string, int> band_cache;                        // shape key -> band
   std::unordered_map<std::string, int> tev_cache;                         // shape key -> screening tile width
   std::unordered_map<std::string, bool> pair_cache;                       // shape key -> 64-sample tiles on CTA pairs
-  bool wide_tiles = true;  // 64-sample tiles for screening / GEMM-only launches of mode banks
+  bool wide_tiles = true;  // 64-sample tiles for screens, and for GEMM-only launches of mode banks
   bool pair_tiles = true;  // those tiles on CTA pairs (single events)
   std::vector<std::unordered_map<std::string, cudaGraphExec_t>> graphs;  // per slot
   double l2_band_bytes = 0;  // extrinsic operand kept in L2 per sweep of the bank
@@ -538,9 +538,9 @@ static int event_alloc(dotpe_ctx *ctx, Event &e, cudaStream_t st, EventRun &R) {
     if (encode_tmap_kblocks(&W.mapB, dt, pa.gpack, b_rows, b.Kpad / 64, (uint64_t)b.Kpad * 2, 2 * TC_TE,
                             tc_kblocks_per_stage()))
       return fail(DOTPE_E_DEVICE, "cuTensorMapEncodeTiled failed (extrinsic operand)");
-    // 128-row boxes for 64-sample tiles (mode banks)
-    if (b.n_pol != 2 && encode_tmap_kblocks(&W.mapB64, dt, pa.gpack, b_rows, b.Kpad / 64, (uint64_t)b.Kpad * 2,
-                                            4 * TC_TE, tc_kblocks_per_stage()))
+    // 128-row boxes for 64-sample tiles
+    if (encode_tmap_kblocks(&W.mapB64, dt, pa.gpack, b_rows, b.Kpad / 64, (uint64_t)b.Kpad * 2, 4 * TC_TE,
+                            tc_kblocks_per_stage()))
       return fail(DOTPE_E_DEVICE, "cuTensorMapEncodeTiled failed (extrinsic operand, 128-row boxes)");
     W.n_etile = L.n_etile;
     W.band = event_band(ctx, e, L, prec_split(e.prec));
@@ -654,12 +654,18 @@ static EpiParams refine_params(const EventRun &R) {
 static std::string band_key(const Event &e, const ScratchLayout &L, bool split);
 
 // Tile width of a single-pass launch: 64-sample tiles where the launch writes
-// no marginal partials (a screening pass with the cut on, or GEMM-only) over a
-// mode bank, unless the context asks for 32-sample tiles; the autotuner's
-// choice for the shape where it has one.
+// no marginal partials (a screening pass with the cut on, or GEMM-only of a mode
+// bank), unless the context asks for 32-sample tiles; the autotuner's choice for the
+// shape where it has one.  A polarisation-resolved bank has no tensor-core <h|h> bound:
+// its wide screen forms each pair's bound while the tile's MMAs run, and is bound by those
+// (16,384 rows x 4,096 samples, 3 detectors, K = 2,048: 2.10 ms, against 3.32 ms in
+// 32-sample tiles, whose operand loads bound it; the whole event 4.08 -> 2.94 ms).
+static bool wide_form(dotpe_ctx *ctx, const Event &e, const EpiParams &P, bool split) {
+  if (!ctx->wide_tiles || split || P.lnl_tile) return false;
+  return P.gemm_only ? e.bank->n_pol != 2 : P.screen_ml && (e.bank->n_pol != 2 || !prec_bf16(e.prec));
+}
 static int launch_tev(dotpe_ctx *ctx, const Event &e, const ScratchLayout &L, const EpiParams &P, bool split) {
-  if (!ctx->wide_tiles || split || e.bank->n_pol == 2 || P.lnl_tile) return 32;
-  if (!(P.gemm_only || P.screen_ml)) return 32;
+  if (!wide_form(ctx, e, P, split)) return 32;
   auto it = ctx->tev_cache.find(band_key(e, L, prec_split(e.prec)));
   return it != ctx->tev_cache.end() ? it->second : 64;
 }
@@ -949,8 +955,7 @@ static int autotune_band(dotpe_ctx *ctx, Event &e, EventRun &R, cudaStream_t st)
   TcWork W = R.W;
   W.P = R.mixed ? screen_params(R) : R.P;
   std::vector<int> tevs{32};
-  if (ctx->wide_tiles && !split_main && e.bank->n_pol != 2 && !W.P.lnl_tile && (W.P.gemm_only || W.P.screen_ml))
-    tevs.push_back(64);
+  if (wide_form(ctx, e, W.P, split_main)) tevs.push_back(64);
   // the 64-sample candidates timed as they run: with the <h|h> bound where the event has it
   if (R.mixed && tevs.back() == 64 && (rc = hh_bound_pass(ctx, e, R, W.P, st)) != DOTPE_OK) return rc;
   const int dflt = tc_band(ctx->l2_band_bytes, e.bank->Kpad / 64, e.bank->M, prec_split(e.prec), R.L.n_etile);

@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(cta_threads(TEV, SCR), 1)
     tc_fused_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ TcBatch<NB> Bt,
                     const TcCommon C) {
   static_assert(SPLIT || !SEP, "a separate low-order accumulator needs split operands");
-  static_assert(TEV == 32 || (TEV == 64 && !SPLIT && HH != 2), "64-sample tiles: single-pass mode banks");
+  static_assert(TEV == 32 || (TEV == 64 && !SPLIT), "64-sample tiles: single pass");
   static_assert(!PAIR || (TEV == 64 && NB == 1), "CTA pairs: 64-sample tiles of one event");
   using PP = Pipe<SPLIT, TEV, PAIR>;
   static_assert(!SCR || (TEV == 32 && !SPLIT), "screens: single pass");
@@ -526,7 +526,8 @@ __global__ void __launch_bounds__(cta_threads(TEV, SCR), 1)
       // <h|h> at every phase that pair_bound uses, C_0 - 2 sum_delta |C_delta|
       // (Eq. hh_ieo), formed while the MMAs of the tile run
       // (a rolled loop into a per-thread array that lives in local memory: small
-      // code, no register pressure, read back once per pair in pass 1)
+      // code, no register pressure, read back once per pair in pass 1; a
+      // polarisation-resolved bank's 63 record floats are held through this loop only)
       float hl[TEV == 64 ? TEV / 2 : 1];
       if constexpr (TEV == 64) {
         if (!P.gemm_only && P.hmin) {
@@ -781,9 +782,10 @@ __global__ void __launch_bounds__(cta_threads(TEV, SCR), 1)
               const int owner = tag >> 8, el = tag & 255;
               if (act) {
                 const int64_t io = (int64_t)it * TI + quad * 32 + owner;
-                const float *mrow = P.mx + io * P.n_det * REC;
+                const float *mrow = P.mx + io * P.n_det * (HH == 2 ? REC_P : REC);
                 float C0, Cr[3], Ci[3];
-                hh_coeffs_by<HH == 1>([&](int q) { return __ldg(mrow + q); }, &T.qs[el * MAXD * REC], P, C0, Cr, Ci);
+                if constexpr (HH == 2) hh_coeffs_pol(mrow, &T.qs[el * MAXD * REC], P, C0, Cr, Ci);
+                else hh_coeffs_by<HH == 1>([&](int q) { return __ldg(mrow + q); }, &T.qs[el * MAXD * REC], P, C0, Cr, Ci);
                 float Zr[MAXM], Zi[MAXM];
 #pragma unroll
                 for (int k = 0; k < MAXM; ++k) {
@@ -1294,14 +1296,15 @@ cudaError_t launch_tc_variant(const TcLaunch &L, const TcBatch<NB> &bt, int grid
   // screens are fp16 passes: no bf16 instantiation of SCR
   constexpr bool BF = !SCR;
   const bool bf16 = BF && L.bf16;
-  if (L.pol) {
-    // polarisation-resolved banks run one event per launch, in 32-sample tiles
+  if (L.pol && TEV == 32) {
+    // polarisation-resolved banks run one event per launch
     if constexpr (NB == 1 && TEV == 32)
       return bf16 ? go(tc_fused_kernel<BF, 2, SPLIT, NB, SEP, TEV, false, SCR>)
                   : go(tc_fused_kernel<false, 2, SPLIT, NB, SEP, TEV, false, SCR>);
     else
       return cudaErrorInvalidValue;
   }
+  if (L.pol && (NB != 1 || L.bf16)) return cudaErrorInvalidValue;  // 64-sample tiles: their fp16 screen
   if constexpr (NB == 1 && TEV == 64 && !SPLIT) {
     if (L.pair) {
       // clusters of two CTAs (grid even)
@@ -1338,12 +1341,15 @@ cudaError_t launch_tc_variant(const TcLaunch &L, const TcBatch<NB> &bt, int grid
         return cudaGetLastError();
       };
       if (grid % 2 != 0) return cudaErrorInvalidValue;
+      if (L.pol) return go2(tc_fused_kernel<false, 2, false, 1, false, 64, true>);
       if (L.bf16) return L.consec ? go2(tc_fused_kernel<true, 1, false, 1, false, 64, true>)
                                   : go2(tc_fused_kernel<true, 0, false, 1, false, 64, true>);
       return L.consec ? go2(tc_fused_kernel<false, 1, false, 1, false, 64, true>)
                       : go2(tc_fused_kernel<false, 0, false, 1, false, 64, true>);
     }
   }
+  if constexpr (NB == 1 && TEV == 64 && !SPLIT)
+    if (L.pol) return go(tc_fused_kernel<false, 2, false, 1, false, 64>);
   if (bf16) return L.consec ? go(tc_fused_kernel<BF, 1, SPLIT, NB, SEP, TEV, false, SCR>)
                             : go(tc_fused_kernel<BF, 0, SPLIT, NB, SEP, TEV, false, SCR>);
   return L.consec ? go(tc_fused_kernel<false, 1, SPLIT, NB, SEP, TEV, false, SCR>)
@@ -1354,7 +1360,7 @@ template <int NB>
 cudaError_t launch_tc_any(const TcLaunch &L, const TcBatch<NB> &bt, int grid, cudaStream_t st) {
   if (L.tev == 64) {
     // 64-sample work tiles: single pass, grid order only (no device list)
-    if (L.split || L.pol || bt.glist) return cudaErrorInvalidValue;
+    if (L.split || bt.glist) return cudaErrorInvalidValue;
     return launch_tc_variant<NB, false, false, 64>(L, bt, grid, st);
   }
   if (!L.split) {

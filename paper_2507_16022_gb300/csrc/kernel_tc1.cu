@@ -10,7 +10,7 @@ int launch_tc_single(const TcLaunch &L, const TcWork *works, const int2 *glist, 
   const int tev = L.tev == 64 ? 64 : 32;
   // CTA pairs: 64-sample tiles in grid order; each CTA loads half of the tile's
   // extrinsic rows, so through the 64-row boxes of the 32-sample map
-  const bool pair = L.pair && tev == 64 && !glist && !L.split && !L.pol;
+  const bool pair = L.pair && tev == 64 && !glist && !L.split;
   TcLaunch Lp = L;
   Lp.pair = pair;
   TcBatch<1> bt;

@@ -122,7 +122,7 @@ struct TcLaunch {
   bool bf16, split, consec;
   bool pol;          // polarisation-resolved bank (row records in registers, n_det <= POL_TC_MAXD)
   bool sep;          // split: hi*lo + lo*hi in their own accumulator (see kernel_tc.cuh)
-  int tev;           // extrinsic samples per work tile: 32, or 64 (single-pass mode banks, grid order)
+  int tev;           // extrinsic samples per work tile: 32, or 64 (single pass, grid order)
   bool pair;         // 64-sample tiles of one event: CTA pairs (cta_group::2, M = 256)
   const int *gate;   // optional device words per event: event k's items run only if gate[k] == gate_want
   int gate_want;
