@@ -80,8 +80,7 @@ SCREEN_TRAFFIC = {"bytes": 0.504e9 + 3.688e9, "n_int": 65536, "n_ext": 4096,
 # of a polarisation-resolved bank (presel_pol_kernel<true>), from one ncu capture:
 # the build it was taken on, its shape and rows.  None = no capture of the current
 # kernel (the figure goes stale with any change to the kernel or its grid).
-PRESEL_TRAFFIC = {"bytes": 1.643e9 + 0.017e9, "rows": 65536, "D": 3, "N_t": 128, "B": 378,
-                  "source": "profiles/presel_pol_rb_fp32_65536x3x128x32.md"}
+PRESEL_TRAFFIC = {"bytes": None, "rows": 65536, "D": 3, "N_t": 128, "B": 378, "source": None}
 
 
 def presel_traffic(simt, rb, D, NT, B, I):
@@ -463,9 +462,10 @@ def bench_batch64(args, dp, ctx_factory, torch, dev, load_peaks_fn):
                      "peak_source": f"{peak_src} bf16_tflops_sustained"},
         "e2e": {"value": pairs * args.steps / (e2e_ms * 1e-3), "unit": "pairs/s", "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": 96 * 64},
-        # per batch: each event's preparation (5) and reduction (6), the batch's fused
-        # launches (mixed: screen, 3 selection kernels, 2 gated refinement variants)
-        "gpu_launches": (64 * (5 + 6) + (6 if args.precision == "mixed" else 1)) * args.steps, "clocks": clocks,
+        # per batch: each event's preparation (5) and reduction (7), and at least one set of
+        # fused launches (mixed: screen, 3 selection kernels, 2 gated refinement variants;
+        # events large enough for launches of their own add theirs)
+        "gpu_launches": (64 * (5 + 7) + (6 if args.precision == "mixed" else 1)) * args.steps, "clocks": clocks,
         "cpu_baseline": None,
     }
     dp.dotpe_bank_release(ctx, bid)
@@ -598,7 +598,7 @@ def bench_presel(args, dp, ctx_factory, torch, dev):
                 "h2d_bytes_per_step": int((rbw[0].nbytes + rbw[1].nbytes) if rbw else
                                           (wl.event.psd.nbytes + wl.event.data.nbytes)) + int(ps.t_grid.nbytes),
                 "d2h_bytes_per_step": int(8 * I + 8 * r["n_selected"] + 64)},
-        "gpu_launches": 6 * args.steps, "clocks": clocks, "cpu_baseline": cpu,
+        "gpu_launches": 7 * args.steps, "clocks": clocks, "cpu_baseline": cpu,
     }
     dp.dotpe_bank_release(ctx, bid)
     dp.dotpe_destroy(ctx)
@@ -740,10 +740,10 @@ def bench_rb(args, dp, ctx_factory, torch, dev):
                 "h2d_bytes_per_step": int(rw.f_fine.nbytes + rw.dff.nbytes + rw.psd_fine.nbytes + rw.data_fine.nbytes
                                           + rw.h0_fine.nbytes + rw.ext.t.nbytes + resp.nbytes + rw.ext.ln_w.nbytes),
                 "d2h_bytes_per_step": int(wdh.nbytes + whh.nbytes + 96)},
-        # per step: the weights kernel; the event's preparation (prep_bins, rb_norm, prep_ext,
+        # per step: the 2 weights kernels; the event's preparation (prep_bins, rb_norm, prep_ext,
         # build_G, pack_G), the fused launches (mixed: screen, 3 selection kernels, 2 gated
-        # refinement variants) and the reduction (6)
-        "gpu_launches": (1 + 5 + (6 if mixed else 1) + 6) * args.steps, "clocks": clocks, "cpu_baseline": cpu,
+        # refinement variants) and the reduction (7)
+        "gpu_launches": (2 + 5 + (6 if mixed else 1) + 7) * args.steps, "clocks": clocks, "cpu_baseline": cpu,
     }
     dp.dotpe_bank_release(ctx, bid)
     dp.dotpe_destroy(ctx)
@@ -883,9 +883,9 @@ def bench_precessing(args, dp, ctx_factory, torch, dev):
                                           + wl.ext.F.nbytes + wl.ext.ln_w.nbytes),
                 "d2h_bytes_per_step": 96},
         # prep (data weights, norm, extrinsic, G build, G pack), the fused kernel (mixed:
-        # screen, 3 selection kernels, 2 gated refinement variants), the reduction (6);
+        # screen, 3 selection kernels, 2 gated refinement variants), the reduction (7);
         # the bank's cross terms are cached from the warm-up
-        "gpu_launches": (5 + (6 if mixed else 1) + 6) * args.steps, "clocks": clocks, "cpu_baseline": cpu,
+        "gpu_launches": (5 + (6 if mixed else 1) + 7) * args.steps, "clocks": clocks, "cpu_baseline": cpu,
     }
     dp.dotpe_bank_release(ctx, bid)
     dp.dotpe_destroy(ctx)
@@ -943,8 +943,8 @@ def bench_pipeline(args, dp, ctx_factory, torch, dev):
         "e2e": {"value": 1.0 / dt, "unit": "events/s", "h2d_bytes_per_step": int(wl.event.psd.nbytes * 2
                 + wl.event.data.nbytes * 2 + ps.t_grid.nbytes + wl.ext.t.nbytes + wl.ext.R.nbytes
                 + wl.ext.ln_w.nbytes), "d2h_bytes_per_step": int(8 * kept[-1] + 96 + 64)},
-        # pre-selection 6, subset 3-5 gathers, coherent event 17 (mixed)
-        "gpu_launches": 28 * args.steps, "clocks": clocks, "cpu_baseline": None,
+        # pre-selection 7, subset 3-5 gathers, coherent event 18 (mixed)
+        "gpu_launches": 30 * args.steps, "clocks": clocks, "cpu_baseline": None,
     }
 
 
@@ -1019,7 +1019,8 @@ def bench_samples(args, dp, ctx_factory, torch, dev):
                                                  "copied between host and device inside)"},
         "roofline": None, "e2e": {"value": n / dt, "unit": "samples/s", "h2d_bytes_per_step": 32 * n,
                                   "d2h_bytes_per_step": 28 * n},
-        "gpu_launches": 2 * args.steps, "clocks": clocks, "cpu_baseline": cpu,
+        # row maximum, sums and prefix, (mode banks' quadrature) weights, draws
+        "gpu_launches": 5 * args.steps, "clocks": clocks, "cpu_baseline": cpu,
     }
 
 
@@ -1442,9 +1443,9 @@ def main():
                and (I, E) == (SCREEN_TRAFFIC["n_int"], SCREEN_TRAFFIC["n_ext"]) else None)
     # prep (data norm, bins, extrinsic, G build, G pack), fused (mixed: <h|h> bound
     # pass of 3 kernels, screen, 3 selection kernels, 2 gated refinement variants),
-    # reduction (2 line, 2 pass, merge, final); cross terms are computed once per
+    # reduction (2 line, 2 pass, merge, marginals, record); cross terms are computed once per
     # (bank, PSD) and reused
-    launches_per_event = 5 + (9 if mixed else 1) + 6
+    launches_per_event = 5 + (9 if mixed else 1) + 7
     dlnz = max(abs(evs[k]["ln_z"] - ref_fp32[k % len(events)][0]["ln_z"]) for k in range(len(evs)))
     if rank != 0:
         if dist is not None:
