@@ -656,16 +656,27 @@ static std::string band_key(const Event &e, const ScratchLayout &L, bool split);
 // Tile width of a single-pass launch: 64-sample tiles where the launch writes
 // no marginal partials (a screening pass with the cut on, or GEMM-only of a mode
 // bank), unless the context asks for 32-sample tiles; the autotuner's choice for the
-// shape where it has one.  A polarisation-resolved bank has no tensor-core <h|h> bound:
-// its wide screen forms each pair's bound while the tile's MMAs run, and is bound by those
-// (16,384 rows x 4,096 samples, 3 detectors, K = 2,048: 2.10 ms, against 3.32 ms in
-// 32-sample tiles, whose operand loads bound it; the whole event 4.08 -> 2.94 ms).
-static bool wide_form(dotpe_ctx *ctx, const Event &e, const EpiParams &P, bool split) {
+// shape where it has one.
+// A polarisation-resolved bank has no tensor-core <h|h> bound: its wide screen forms each
+// pair's bound while the tile's MMAs run, and is bound by those (16,384 rows x 4,096
+// samples, 3 detectors, K = 2,048: 2.10 ms, against 3.32 ms in 32-sample tiles, whose
+// operand loads bound it; the whole event 4.08 -> 2.94 ms).  But each CTA's first tile has
+// no threshold yet and evaluates all of its pairs out of the pool, ~0.1 ms whatever the
+// event's size, which the 32-sample epilogue does in place: wide from POL_WIDE_STEPS k-block
+// steps per SM.  Events, wide against narrow: 4,096 x 2,048, 4 modes, K = 2,048 (1,725 steps)
+// 0.80 and 0.86 ms; 16,384 x 256, K = 1,024 (431 steps) 0.50 and 0.43; 2,048 x 512 (108
+// steps) 0.41 and 0.33; 300 x 77 0.34 and 0.23.
+constexpr int64_t POL_WIDE_STEPS = 1500;  // 128 x 32-pair tiles x modes x k-blocks of 64, per SM
+static bool wide_form(dotpe_ctx *ctx, const Event &e, const ScratchLayout &L, const EpiParams &P, bool split) {
   if (!ctx->wide_tiles || split || P.lnl_tile) return false;
-  return P.gemm_only ? e.bank->n_pol != 2 : P.screen_ml && (e.bank->n_pol != 2 || !prec_bf16(e.prec));
+  const Bank &b = *e.bank;
+  if (b.n_pol != 2) return P.gemm_only || P.screen_ml;
+  if (P.gemm_only || !P.screen_ml || prec_bf16(e.prec)) return false;
+  const int64_t tiles = (P.n_int + TC_TI - 1) / TC_TI * L.n_etile;
+  return tiles * b.M * (b.Kpad / 64) >= POL_WIDE_STEPS * ctx->n_sms;
 }
 static int launch_tev(dotpe_ctx *ctx, const Event &e, const ScratchLayout &L, const EpiParams &P, bool split) {
-  if (!wide_form(ctx, e, P, split)) return 32;
+  if (!wide_form(ctx, e, L, P, split)) return 32;
   auto it = ctx->tev_cache.find(band_key(e, L, prec_split(e.prec)));
   return it != ctx->tev_cache.end() ? it->second : 64;
 }
@@ -955,7 +966,7 @@ static int autotune_band(dotpe_ctx *ctx, Event &e, EventRun &R, cudaStream_t st)
   TcWork W = R.W;
   W.P = R.mixed ? screen_params(R) : R.P;
   std::vector<int> tevs{32};
-  if (wide_form(ctx, e, W.P, split_main)) tevs.push_back(64);
+  if (wide_form(ctx, e, R.L, W.P, split_main)) tevs.push_back(64);
   // the 64-sample candidates timed as they run: with the <h|h> bound where the event has it
   if (R.mixed && tevs.back() == 64 && (rc = hh_bound_pass(ctx, e, R, W.P, st)) != DOTPE_OK) return rc;
   const int dflt = tc_band(ctx->l2_band_bytes, e.bank->Kpad / 64, e.bank->M, prec_split(e.prec), R.L.n_etile);

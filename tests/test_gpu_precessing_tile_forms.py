@@ -1,5 +1,5 @@
 """The screen of a polarisation-resolved bank in its three tile forms: 64-sample tiles on CTA
-pairs (the default), on one SM each, and 32-sample tiles.  Ragged rows and samples, an odd
+pairs (the default for large events), on one SM each, and 32-sample tiles.  Ragged rows and samples, an odd
 number of 32-sample tiles and of bank tiles, a shape large enough for pilot tiles, one to
 four modes and one to three detectors, odd k-blocks.
 
@@ -42,7 +42,9 @@ def _run(dp, ctx, wl, precision):
 
 
 @pytest.mark.parametrize("shape", [(1, 1, 3, 4, 64), (129, 33, 1, 1, 96), (300, 77, 2, 3, 128), (513, 97, 3, 2, 200),
-                                   (257, 128, 3, 4, 250), (2100, 1000, 3, 4, 128)],
+                                   (257, 128, 3, 4, 250), (2100, 1000, 3, 4, 128),
+                                   # enough work for the 64-sample tiles (the shapes above stay narrow)
+                                   (4033, 2017, 3, 4, 490), (6200, 2399, 2, 2, 510), (8201, 3521, 1, 1, 512)],
                          ids=lambda s: "x".join(map(str, s)))
 def test_forms_agree(forms, shape):
     import oracle
