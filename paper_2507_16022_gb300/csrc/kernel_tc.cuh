@@ -565,18 +565,22 @@ __global__ void __launch_bounds__(cta_threads(TEV, SCR), 1)
       bool skip = false, have_c = false;
       float cf[TcTail::GEN ? EHALF : 1][8];
       uint2 hw[2] = {make_uint2(0u, 0u), make_uint2(0u, 0u)};
+      // the tile's sample of this thread's pair j (SEP: of the first 16-sample half, then of the second)
+      auto sample_of = [&](int j) {
+        return SEP ? (16 * (j / (EHALF / 2)) + (EHALF / 2) * half + j % (EHALF / 2)) : (half * EHALF + j);
+      };
       if constexpr (TcTail::GEN) {
         skip = thr > 0.f && !store && !P.gemm_only && !P.screen_ml;
         have_c = !(skip && P.hmin) && !P.gemm_only;
+        // (each warp presets the entries of its own pairs: no barrier stands before their values)
 #pragma unroll
-        for (int j = 0; j < EHALF; ++j) T.xs[row * XS_LD + half * EHALF + j] = -INFINITY;
+        for (int j = 0; j < EHALF; ++j) T.xs[row * XS_LD + sample_of(j)] = -INFINITY;
         if (have_c) {
           load_mrec();
 #pragma unroll 1
           for (int j = 0; j < EHALF; ++j) {
-            const int el = SEP ? (16 * (j / (EHALF / 2)) + (EHALF / 2) * half + j % (EHALF / 2)) : (half * EHALF + j);
             float C0, Cr[3], Ci[3];
-            hh_tile<HH>(mrec, &T.qs[el * MAXD * REC], P, C0, Cr, Ci);
+            hh_tile<HH>(mrec, &T.qs[sample_of(j) * MAXD * REC], P, C0, Cr, Ci);
             float h = C0;
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
@@ -1012,10 +1016,6 @@ __global__ void __launch_bounds__(cta_threads(TEV, SCR), 1)
         Lse rb;
         rb.init();
         int np = 0;
-        auto sample_of = [&](int j) {
-          // SEP: samples of the first 16-sample half, then of the second
-          return SEP ? (16 * (j / (EHALF / 2)) + (EHALF / 2) * half + j % (EHALF / 2)) : (half * EHALF + j);
-        };
         const float zcm = zs * zs * 1.000006f, thr2 = 2.f * thr;
         const bool any_lw = P.lw_int || P.lw_ext;
         float *pz = &T.pz[ew * PAIR_POOL * 2 * MAXM];
