@@ -521,7 +521,9 @@ __global__ void __launch_bounds__(cta_threads(TEV, SCR), 1)
       if constexpr (TcTail::GEN)
         for (int k = etid; k < TEV; k += EPT) T.lwe[k] = (P.lw_ext && e0 + k < P.n_ext) ? P.lw_ext[e0 + k] : 0.0;
       named_bar_sync(1, EPT);
-      float thr = tile_threshold(P);
+      // one lane's reading for the warp: the running maximum may rise between two lanes' loads, and
+      // what the epilogue skips and collects is decided by whole warps
+      float thr = __shfl_sync(0xffffffffu, tile_threshold(P), 0);
       // 64-sample screen: for each of the thread's pairs the lower bound of
       // <h|h> at every phase that pair_bound uses, C_0 - 2 sum_delta |C_delta|
       // (Eq. hh_ieo), formed while the MMAs of the tile run
