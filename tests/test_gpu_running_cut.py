@@ -37,7 +37,7 @@ def test_running_cut_keeps_the_evidence(precision, rows, n_ext, modes):
         for _ in range(10):
             ev = event(40.0)
             assert abs(ev["ln_z"] - ref["ln_z"]) <= 1e-4
-            assert ev["max_lnl_ml"] == pytest.approx(ref["max_lnl_ml"], abs=1e-4)
+            assert ev["max_lnl_ml"] == pytest.approx(ref["max_lnl_ml"], abs=1e-3)
             assert 0 < ev["n_marginalised"] < ref["n_marginalised"]
     finally:
         dp.dotpe_destroy(ctx)
