@@ -2716,6 +2716,8 @@ static int recompute_block(dotpe_ctx *ctx, Event &e, int64_t a, int64_t b, int64
     CUDA_OR_FAIL(cudaStreamSynchronize(st));
     const float *src = (what == DOTPE_LNL_MARG) ? sub.lnl_tile : sub.ml_tile;
     cudaError_t ce = cudaMemcpy2D(out, ld * 4, src, sub.NE * 4, sub.NE * 4, sub.NI, cudaMemcpyDefault);
+    // (a copy within the device returns before it is done, and the block goes back to the pool below)
+    if (ce == cudaSuccess) ce = cudaStreamSynchronize(0);
     if (ce != cudaSuccess) rc = fail(DOTPE_E_DEVICE, "copying the recomputed block: %s", cudaGetErrorString(ce));
   } else {
     cudaStreamSynchronize(st);
