@@ -260,18 +260,23 @@ __device__ __forceinline__ float lnl_ml_of(float dh, float hh) {
   return (dh > 0.f && hh > 0.f) ? __fdividef(0.5f * dh * dh, hh) : 0.f;
 }
 
-// Online sums of exp(l) and exp(2 l) over N more values.
+// The maximum as the sums' reference: finite also where nothing has been added yet (-inf,
+// whose terms are then zero) and where a value has overflowed (its sum stays +inf).
+__device__ __forceinline__ float lse_ref(float m) { return fminf(fmaxf(m, -3.402823466e38f), 3.402823466e38f); }
+
+// Online sums of exp(l) and exp(2 l) over N more values (-inf: none).
 template <int N>
 __device__ __forceinline__ void lse2_add(float &mx, float &s1, float &s2, const float (&l)[N]) {
   float m = mx;
 #pragma unroll
   for (int k = 0; k < N; ++k) m = fmaxf(m, l[k]);
-  const float r = __expf(mx - m);
+  const float c = lse_ref(m);
+  const float r = __expf(mx - c);
   s1 *= r;
   s2 *= r * r;
 #pragma unroll
   for (int k = 0; k < N; ++k) {
-    const float q = __expf(l[k] - m);
+    const float q = __expf(l[k] - c);
     s1 += q;
     s2 = fmaf(q, q, s2);
   }
@@ -291,12 +296,10 @@ struct PhaseSums {
                 o2 = __shfl_xor_sync(0xffffffffu, s2, o), ob = __shfl_xor_sync(0xffffffffu, best, o);
     const int oa = __shfl_xor_sync(0xffffffffu, argo, o);
     npass += __shfl_xor_sync(0xffffffffu, npass, o);
-    const float m = fmaxf(mx, om);
-    if (m > -INFINITY) {
-      const float r = __expf(mx - m), q = __expf(om - m);
-      s1 = fmaf(s1, r, o1 * q);
-      s2 = fmaf(s2, r * r, o2 * q * q);
-    }
+    const float m = fmaxf(mx, om), c = lse_ref(m);
+    const float r = __expf(mx - c), q = __expf(om - c);
+    s1 = fmaf(s1, r, o1 * q);
+    s2 = fmaf(s2, r * r, o2 * q * q);
     mx = m;
     if (ob > best || (ob == best && oa < argo)) { best = ob; argo = oa; }
   }
@@ -311,27 +314,45 @@ struct PhaseSums {
   }
 };
 
+// phase_quad's sums differ from phase_at's by the order of their additions and the entries
+// of the phase table that they start from: by less than 2^-18 of sum |Z| and of
+// C_0 + 2 sum |C_delta| (the entries agree to 5e-7, each sum rounds at most 8 times).
+constexpr float PHASE_SLACK = 3.8146973e-6f;
+
 // One pair over the phase grid, or the part of it with base phases b0, b0 + step, ...
-// Phases go four at a time (a quarter turn apart when n_phi is a multiple of 4, else
-// phase by phase).  Without a cut (thr <= 0: every phase has ln L^ML >= 0) all are
-// marginalised as they come, two gathers of the distance table in flight.  With one, the
-// phases that pass are marked first, by dh > 0 and dh^2 >= 2 thr hh, and then
-// marginalised two at a time, each thread taking its own next ones: a warp takes as
-// many steps as its busiest lane has passing phases, not one for every phase that any of
-// its lanes passes.  ln L^ML itself is needed for the phases that pass only (the maximum
-// is among them), or with want_best for all.
+// Without a cut (thr <= 0: every phase has ln L^ML >= 0) phases go four at a time (a
+// quarter turn apart when n_phi is a multiple of 4, else phase by phase) and all are
+// marginalised as they come, two gathers of the distance table in flight.
+// With a cut a phase is kept where its ln L^ML, from phase_at, reaches thr: one decision
+// for every kernel, grid and option, so that an event keeps the same phases whichever way
+// its pairs are evaluated.  The phases that may pass are marked first, four at a time, by
+// dh > 0 and dh^2 >= 2 thr hh with the slack of the quick sums, and then evaluated two at a
+// time, each thread taking its own next ones: a warp takes as many steps as its busiest
+// lane has marked phases, not one for every phase that any of its lanes passes.  ln L^ML
+// itself is needed for those only (the maximum is among them), or with want_best (stored
+// values) for all phases, which then go through phase_at one by one.
 __device__ __forceinline__ void pair_phases(const float (&Zr)[4], const float (&Zi)[4], float C0,
                                             const float (&Cr)[3], const float (&Ci)[3], float thr, bool want_best,
                                             const EpiParams &P, const float4 *__restrict__ ph, int b0, int step,
                                             PhaseSums &S) {
   const int n = P.n_phi, nb = (n + 3) >> 2;
-  const bool quad = (n & 3) == 0, all = !(thr > 0.f);
+  const bool quad = (n & 3) == 0, all = !(thr > 0.f), exact = !quad || (want_best && !all);
   const float thr2 = 2.f * thr;
-  uint32_t mk[4] = {0u, 0u, 0u, 0u};  // bit b of mk[j]: phase b + j nb passes (nb <= 32)
+  float dh_slack = 0.f, hh_slack = 0.f;
+  if (!exact) {
+    float a = 0.f, h = fabsf(C0);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a += fabsf(Zr[k]) + fabsf(Zi[k]);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) h += 2.f * (fabsf(Cr[k]) + fabsf(Ci[k]));
+    dh_slack = PHASE_SLACK * a;
+    hh_slack = PHASE_SLACK * h * thr2;
+  }
+  uint32_t mk[4] = {0u, 0u, 0u, 0u};  // bit b of mk[j]: phase b + j nb may pass (nb <= 32)
 #pragma unroll 1
   for (int b = b0; b < nb; b += step) {
     float dh[4], hh[4];
-    if (quad) {
+    if (!exact) {
       phase_quad(Zr, Zi, C0, Cr, Ci, ph, b, dh, hh);
     } else {
 #pragma unroll
@@ -349,11 +370,14 @@ __device__ __forceinline__ void pair_phases(const float (&Zr)[4], const float (&
         if (on && (ml > S.best || (ml == S.best && o < S.argo))) { S.best = ml; S.argo = o; }
         mk[j] |= (on && ml >= thr) ? 1u << b : 0u;
       }
+    } else if (exact) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) mk[j] |= lnl_ml_of(dh[j], hh[j]) >= thr ? 1u << b : 0u;
     } else {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const float r = thr2 * hh[j];
-        mk[j] |= (dh[j] * fmaxf(dh[j], 0.f) >= r && r > 0.f) ? 1u << b : 0u;
+        const float d = fmaxf(dh[j] + dh_slack, 0.f);
+        mk[j] |= d * d >= fmaf(thr2, hh[j], -hh_slack) ? 1u << b : 0u;
       }
     }
     if (all) {
@@ -373,8 +397,10 @@ __device__ __forceinline__ void pair_phases(const float (&Zr)[4], const float (&
       lse2_add<4>(S.mx, S.s1, S.s2, l);
     }
   }
-  S.npass = __popc(mk[0]) + __popc(mk[1]) + __popc(mk[2]) + __popc(mk[3]);
-  if (all) return;
+  if (all) {
+    S.npass = __popc(mk[0]) + __popc(mk[1]) + __popc(mk[2]) + __popc(mk[3]);
+    return;
+  }
   // up to 32 phases in one word, else a word per quarter of the grid
   const bool one = nb <= 8;
   if (one) mk[0] |= (mk[1] << 8) | (mk[2] << 16) | (mk[3] << 24);
@@ -394,14 +420,15 @@ __device__ __forceinline__ void pair_phases(const float (&Zr)[4], const float (&
       float dh[2], hh[2], l[2];
       phase_at(Zr, Zi, C0, Cr, Ci, ph, o0, dh[0], hh[0]);
       phase_at(Zr, Zi, C0, Cr, Ci, ph, o1, dh[1], hh[1]);
-      if (!want_best) {
-        // (in increasing o: the lowest keeps a tie)
-        const float m0 = lnl_ml_of(dh[0], hh[0]), m1 = lnl_ml_of(dh[1], hh[1]);
-        if (m0 > S.best) { S.best = m0; S.argo = o0; }
-        if (m1 > S.best) { S.best = m1; S.argo = o1; }
-      }
+      const float m0 = lnl_ml_of(dh[0], hh[0]), m1 = lnl_ml_of(dh[1], hh[1]);
+      // (in increasing o: the lowest keeps a tie)
+      if (m0 > S.best) { S.best = m0; S.argo = o0; }
+      if (m1 > S.best) { S.best = m1; S.argo = o1; }
+      const bool k0 = m0 >= thr, k1 = two && m1 >= thr;
+      S.npass += (int)k0 + (int)k1;
       dm_lnlbar_n<2>(dh, hh, P.u_min, P.dm_table, l);
-      if (!two) l[1] = -INFINITY;
+      if (!k0) l[0] = -INFINITY;
+      if (!k1) l[1] = -INFINITY;
       lse2_add<2>(S.mx, S.s1, S.s2, l);
     }
   }
