@@ -406,8 +406,6 @@ struct EventRun {
   TcWork W;
   ReduceArgs ra;
   bool mixed = false;
-  // the current block's <h|h> bound (tensor-core pass), for its screen and refinement
-  const __nv_bfloat16 *hmin = nullptr;
 };
 
 // The bank operand map and the shape common to every event of a launch.
@@ -646,8 +644,6 @@ static EpiParams refine_params(const EventRun &R) {
   EpiParams Pf = R.P;
   Pf.ml_running = (float *)(R.scr + R.L.ml_refine);
   Pf.track_max = 0;
-  Pf.hmin = R.hmin;
-  Pf.hmin_ld = R.hmin ? hb_ld(R.P.n_ext) : 0;
   return Pf;
 }
 
@@ -691,7 +687,7 @@ static bool launch_pair(dotpe_ctx *ctx, const Event &e, const ScratchLayout &L) 
 
 // The <h|h> bound of every pair of the current bank block on the tensor cores,
 // for the 64-sample screen P (when the event's scratch has room for it).
-static int hh_bound_pass(dotpe_ctx *ctx, const Event &e, EventRun &R, EpiParams &P, cudaStream_t st) {
+static int hh_bound_pass(dotpe_ctx *ctx, const Event &e, const EventRun &R, EpiParams &P, cudaStream_t st) {
   if (R.L.hb_bytes == 0) return DOTPE_OK;
   HbDelta dl;
   for (int p = 0; p < NPAIR; ++p) dl.pdelta[p] = R.P.pdelta[p];
@@ -699,7 +695,6 @@ static int hh_bound_pass(dotpe_ctx *ctx, const Event &e, EventRun &R, EpiParams 
   if (launch_hh_bound(R.P.n_int, e.NE, e.D, dl, R.P.mx, R.pa.qx, R.scr + R.L.hb, &hmin, ctx->n_sms, R.P.status,
                       st) != 0)
     return fail(DOTPE_E_DEVICE, "<h|h> bound launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-  R.hmin = hmin;
   P.hmin = hmin;
   P.hmin_ld = hb_ld(e.NE);
   return DOTPE_OK;

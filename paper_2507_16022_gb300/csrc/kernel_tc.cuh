@@ -560,24 +560,25 @@ __global__ void __launch_bounds__(cta_threads(TEV, SCR), 1)
         }
       }
       // General epilogue.  With a cut and nothing stored a pair is skipped where an upper
-      // bound of its ln L^ML is below the threshold: the bound's <h|h> comes from the
-      // tensor-core pass where the event has it (the sum over modes is then all that a
-      // skipped pair costs), else from the pair's own coefficients.  Those, where every pair
-      // needs them, are formed here, while the tile's MMAs run, into a per-thread array.
-      bool skip = false, have_c = false;
+      // bound of its ln L^ML is below the threshold.  The pairs' <h|h> coefficients and their
+      // lower bounds are formed here, while the tile's MMAs run, into a per-thread array.
+      // The screen's tensor-core bound is not read here, although it would skip most pairs
+      // sooner (a batch of 12 events over 65,536 rows 65.9 against 68.2 ms, relative binning
+      // 32,768 x 2,048 7.3 against 7.8 ms): which pairs are left decides how they are
+      // evaluated, so an event's last bits would follow from whether its screen had the
+      // memory and the tile form for that bound.
+      bool skip = false;
       float cf[TcTail::GEN ? EHALF : 1][8];
-      uint2 hw[2] = {make_uint2(0u, 0u), make_uint2(0u, 0u)};
       // the tile's sample of this thread's pair j (SEP: of the first 16-sample half, then of the second)
       auto sample_of = [&](int j) {
         return SEP ? (16 * (j / (EHALF / 2)) + (EHALF / 2) * half + j % (EHALF / 2)) : (half * EHALF + j);
       };
       if constexpr (TcTail::GEN) {
         skip = thr > 0.f && !store && !P.gemm_only && !P.screen_ml;
-        have_c = !(skip && P.hmin) && !P.gemm_only;
         // (each warp presets the entries of its own pairs: no barrier stands before their values)
 #pragma unroll
         for (int j = 0; j < EHALF; ++j) T.xs[row * XS_LD + sample_of(j)] = -INFINITY;
-        if (have_c) {
+        if (!P.gemm_only) {
           load_mrec();
 #pragma unroll 1
           for (int j = 0; j < EHALF; ++j) {
@@ -593,24 +594,12 @@ __global__ void __launch_bounds__(cta_threads(TEV, SCR), 1)
             cf[j][0] = C0;
             cf[j][7] = h;
           }
-        } else if (skip) {
-          const int64_t ib = vi ? i : 0;
-          const __nv_bfloat16 *src = P.hmin + ib * P.hmin_ld + e0;
-#pragma unroll
-          for (int q = 0; q < 2; ++q)
-            hw[q] = __ldg(reinterpret_cast<const uint2 *>(src + (SEP ? 16 * q + 4 * half : EHALF * half + 4 * q)));
         }
       }
       auto coef_of = [&](int j, float &C0, float (&Cr)[3], float (&Ci)[3]) {
         C0 = cf[j][0];
 #pragma unroll
         for (int q = 0; q < 3; ++q) { Cr[q] = cf[j][1 + 2 * q]; Ci[q] = cf[j][2 + 2 * q]; }
-      };
-      auto hlow = [&](int j) -> float {
-        if (have_c) return cf[j][7];
-        const uint2 w2 = j < 4 ? hw[0] : hw[1];
-        const uint32_t w1 = (j & 2) ? w2.y : w2.x;
-        return __uint_as_float((j & 1) ? (w1 & 0xffff0000u) : (w1 << 16));
       };
       // 64-sample screen with three or four modes: modes 0 and 1 complete first;
       // their share of sum_m |Z_m| per pair is read while the other modes' MMAs run
@@ -1079,7 +1068,7 @@ __global__ void __launch_bounds__(cta_threads(TEV, SCR), 1)
               float a = 0.f;
 #pragma unroll
               for (int k = 0; k < MAXM; ++k) a += sqrt_near(fmaf(Zr[k], Zr[k], Zi[k] * Zi[k]));
-              const float h = hlow(j);
+              const float h = cf[j][7];
               mine = mine && !(h > 0.f && zcm * a * a < thr2 * h);
             }
 #pragma unroll
@@ -1121,22 +1110,20 @@ __global__ void __launch_bounds__(cta_threads(TEV, SCR), 1)
               for (int k = 0; k < MAXM; ++k) { zr[k] = Zr[k]; zi[k] = Zi[k]; }
             }
             const int64_t io = (int64_t)it * TI + quad * 32 + own;
-            if (direct && have_c) {
+            if (direct) {
               coef_of(j, C0, Cr, Ci);
             } else {
-              // from the row's record in memory; a collected pair's four lanes take a
-              // detector each and add (the order of the one-lane sum)
-              hh_row<HH>(P.mx, act ? io : (int64_t)0, &T.qs[sm * MAXD * REC], P, direct ? 0 : (lane & 3),
-                         direct ? P.n_det : min(P.n_det, (lane & 3) + 1), C0, Cr, Ci);
-              if (!direct) {
+              // a collected pair's coefficients from its row's record in memory: its four lanes
+              // take a detector each and add (the order of the one-lane sum)
+              hh_row<HH>(P.mx, act ? io : (int64_t)0, &T.qs[sm * MAXD * REC], P, lane & 3, min(P.n_det, (lane & 3) + 1),
+                         C0, Cr, Ci);
 #pragma unroll
-                for (int o = 1; o <= 2; o <<= 1) {
-                  C0 += __shfl_xor_sync(0xffffffffu, C0, o);
+              for (int o = 1; o <= 2; o <<= 1) {
+                C0 += __shfl_xor_sync(0xffffffffu, C0, o);
 #pragma unroll
-                  for (int k = 0; k < 3; ++k) {
-                    Cr[k] += __shfl_xor_sync(0xffffffffu, Cr[k], o);
-                    Ci[k] += __shfl_xor_sync(0xffffffffu, Ci[k], o);
-                  }
+                for (int k = 0; k < 3; ++k) {
+                  Cr[k] += __shfl_xor_sync(0xffffffffu, Cr[k], o);
+                  Ci[k] += __shfl_xor_sync(0xffffffffu, Ci[k], o);
                 }
               }
             }
