@@ -711,7 +711,7 @@ static int event_fused(dotpe_ctx *ctx, Event &e, EventRun &R, bool last_block, c
     sg.I_bank = b.I;
     sg.Kpad = b.Kpad;
     sg.K = 2 * b.n_pol * b.B;
-    launch_simt(sg, R.P, st);
+    launch_simt(sg, R.P, ctx->n_sms, st);
     return DOTPE_OK;
   }
   TcLaunch T;

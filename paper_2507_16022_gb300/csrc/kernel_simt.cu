@@ -21,6 +21,8 @@
 //
 // Epilogue: Z through shared memory (free after the mainloop), then a warp per row and a
 // lane per sample: the row's record is a broadcast, stored values are written in whole lines.
+#include <algorithm>
+
 #include "common.cuh"
 #include "epilogue.cuh"
 #include "kernels.h"
@@ -73,13 +75,13 @@ __device__ __forceinline__ uint64_t fma2(float a, uint64_t b, uint64_t c) {
 __device__ __forceinline__ int z_at(int c, int row, int el) { return c * Z_W + row * TE + (el ^ ((row & 3) << 3)); }
 }  // namespace
 
-__global__ void __launch_bounds__(GT * MAXM, 2) simt_fused_kernel(SimtArgs g, EpiParams P) {
+__global__ void __launch_bounds__(GT * MAXM, 2) simt_fused_kernel(SimtArgs g, EpiParams P, int tile0, int n_etile) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   const int M = P.n_modes;
   float *stage = reinterpret_cast<float *>(smem_raw);
   SimtSmem &S = *reinterpret_cast<SimtSmem *>(smem_raw + stage_bytes(M));
   const int tid = threadIdx.x, nt = blockDim.x;
-  const int et = blockIdx.x, it = blockIdx.y;
+  const int tile = tile0 + (int)blockIdx.x, it = tile / n_etile, et = tile % n_etile;
   const int64_t i0 = (int64_t)it * TI, e0 = (int64_t)et * TE;
   const int m = tid / GT, t = tid % GT;  // this thread's mode
   const int ty = t / 8, tx = t % 8;      // rows ty + 8 r, samples tx + 8 j
@@ -259,7 +261,6 @@ __global__ void __launch_bounds__(GT * MAXM, 2) simt_fused_kernel(SimtArgs g, Ep
       n += S.w_np[q];
       if (S.w_ml[q] > bv || (S.w_ml[q] == bv && S.w_arg[q] < bi)) { bv = S.w_ml[q]; bi = S.w_arg[q]; }
     }
-    const int64_t tile = (int64_t)it * gridDim.x + et;
     P.tile_part[tile] = make_float4(a.m, a.s, b.m, b.s);
     P.tile_ml[tile] = bv;
     P.tile_arg[tile] = bi;
@@ -268,11 +269,23 @@ __global__ void __launch_bounds__(GT * MAXM, 2) simt_fused_kernel(SimtArgs g, Ep
   }
 }
 
-void launch_simt(const SimtArgs &g, const EpiParams &P, cudaStream_t st) {
-  dim3 grid((unsigned)((P.n_ext + TE - 1) / TE), (unsigned)((P.n_int + TI - 1) / TI));
+// A block's cut is the maximum that it finds when its products are done, so what is in flight
+// at first is marginalised whole: two blocks per SM with three or four modes, whose registers
+// fill it.  Of one or two modes more blocks fit, up to all of a small event's (6,456 x 207, two
+// modes, best ln L 36: every phase kept and ln Z 5e-4 higher).  Under a running cut the first two
+// blocks per SM are then a launch of their own, and the others find its maximum; 8,192 x 1,024,
+// B 512, two modes 2.20 ms (2.27 ms in one launch with twice the phases kept).
+constexpr int PILOT_PER_SM = 2;
+
+void launch_simt(const SimtArgs &g, const EpiParams &P, int n_sms, cudaStream_t st) {
+  const int n_etile = (int)((P.n_ext + TE - 1) / TE);
+  const int n = n_etile * (int)((P.n_int + TI - 1) / TI);
+  const size_t smem = stage_bytes(P.n_modes) + sizeof(SimtSmem);
   cudaFuncSetAttribute(simt_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)(stage_bytes(MAXM) + sizeof(SimtSmem)));
-  simt_fused_kernel<<<grid, GT * P.n_modes, stage_bytes(P.n_modes) + sizeof(SimtSmem), st>>>(g, P);
+  const int pilot = (P.track_max && P.n_modes <= 2) ? std::min(n, PILOT_PER_SM * n_sms) : 0;
+  if (pilot > 0) simt_fused_kernel<<<pilot, GT * P.n_modes, smem, st>>>(g, P, 0, n_etile);
+  if (n > pilot) simt_fused_kernel<<<n - pilot, GT * P.n_modes, smem, st>>>(g, P, pilot, n_etile);
 }
 
 }  // namespace dotpe

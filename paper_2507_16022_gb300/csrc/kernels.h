@@ -85,7 +85,7 @@ struct SimtArgs {
   int Kpad, K;      // K = 2B (multiple-of-8 not required)
 };
 constexpr int SIMT_TI = 64, SIMT_TE = 32;
-void launch_simt(const SimtArgs &g, const EpiParams &P, cudaStream_t st);
+void launch_simt(const SimtArgs &g, const EpiParams &P, int n_sms, cudaStream_t st);
 
 // Fused tcgen05 kernel over a batch of events sharing one bank.
 constexpr int TC_TI = 128, TC_TE = 32;
