@@ -338,7 +338,7 @@ typedef struct dotpe_rb_desc {
 /* ---- context ----------------------------------------------------------- */
 /* Creates a context on cfg->device (cfg may be NULL: defaults) and its
  * streams.  The distance-marginal lookup table of Eq. lnl_dist_marginalized
- * lives in static device memory (9 MB per GPU that loads the library, held
+ * lives in static device memory (17 MB per GPU that loads the library, held
  * until the process exits); the first context created in a CUDA context of
  * the device builds it (about 0.1 s of FP64 work), later ones share it.
  * Errors: E_INVALID (bad device), E_DEVICE, E_NOMEM. */

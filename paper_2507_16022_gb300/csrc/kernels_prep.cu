@@ -715,30 +715,33 @@ __global__ void build_dm_table_kernel(float4 *__restrict__ tab) {
 }
 
 // One cell of the polynomial table (see dist_marg.cuh): R and its derivatives at the
-// cell's four nodes, K's from the node table and the rest in closed form (FP64), then
-// the bicubic coefficients of u, v in [0, 1].
+// cell's four corners, K's from the node table's bicubic (at a node, or half way to the
+// next in ln s) and the rest in closed form (FP64), then the bicubic coefficients of u, v
+// in [0, 1].
 __global__ void build_dm_cells_kernel(const float4 *__restrict__ tab, float4 *__restrict__ cells) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= DMC_NY * DMC_NS) return;
   const int iy = k % DMC_NY, is = k / DMC_NY;
+  const double ds = DM_DS / 2.0;  // a cell's step in ln s
   double F[4][4];  // rows: value at u = 0, 1, d/du at u = 0, 1; columns the same in v
   for (int cy = 0; cy < 2; ++cy)
     for (int cs = 0; cs < 2; ++cs) {
-      double y, hy;
-      if (iy < DMC_N0) { hy = 0.125; y = -64.0 + hy * (iy + cy); }
-      else if (iy < DMC_N0 + DMC_N1) { hy = 0.0625; y = hy * (iy - DMC_N0 + cy); }
-      else { hy = 0.125; y = 12.0 + hy * (iy - DMC_N0 - DMC_N1 + cy); }
-      int ny;  // the node table's index of y
-      if (y < -2.0) ny = (int)((y + 64.0) * 8.0 + 0.5);
-      else if (y < 12.0) ny = DM_NA + (int)((y + 2.0) * 32.0 + 0.5);
-      else ny = DM_NA + DM_NB + (int)((y - 12.0) * 8.0 + 0.5);
-      const int ns = DMC_IS0 + is + cs;
-      const float4 q = tab[ns * DM_NY + ny];
-      const double sig = (double)DM_S0 + (double)DM_DS * ns, s = exp(sig), m = mu_d(y);
+      const double y = dm_node_y(iy + cy), hy = dm_node_y(iy + 1) - dm_node_y(iy);
+      const int h = is + cs, ns = DMC_IS0 + h / 2;  // half nodes from DMC_S0, the node at or below
+      const float4 q0 = tab[ns * DM_NY + iy + cy];
+      double K = q0.x, Ky = q0.y, Ks = 0.5 * q0.z, Kys = 0.5 * q0.w;  // ln s derivatives per half step
+      if (h % 2) {
+        const float4 q1 = tab[(ns + 1) * DM_NY + iy + cy];
+        K = 0.5 * ((double)q0.x + q1.x) + 0.125 * ((double)q0.z - q1.z);
+        Ky = 0.5 * ((double)q0.y + q1.y) + 0.125 * ((double)q0.w - q1.w);
+        Ks = 0.75 * ((double)q1.x - q0.x) - 0.125 * ((double)q0.z + q1.z);
+        Kys = 0.75 * ((double)q1.y - q0.y) - 0.125 * ((double)q0.w + q1.w);
+      }
+      const double sig = (double)DMC_S0 + ds * h, s = exp(sig), m = mu_d(y);
       const double dm = 0.5 * (1.0 + y / sqrt(y * y + 4.0));
       // T = ln Phi(y) (+ y^2 / 2 on the side y < 0, whose base is s (x - s / 2))
       double T, Ty;
-      if (iy < DMC_N0) {
+      if (dm_node_y(iy) < 0.0) {
         const double ex = erfcx(-y * 0.70710678118654752);
         T = log(0.5 * ex);
         Ty = 0.79788456080286536 / ex + y;
@@ -749,10 +752,10 @@ __global__ void build_dm_cells_kernel(const float4 *__restrict__ tab, float4 *__
       }
       const double C = 1.0986122886681098 + 0.91893853320467274;  // ln 3 + ln(2 pi) / 2
       const double sm = s + m;
-      F[cy][cs] = (double)q.x + T + C + 3.0 * sig - 4.0 * log(sm);
-      F[2 + cy][cs] = hy * ((double)q.y + Ty - 4.0 * dm / sm);
-      F[cy][2 + cs] = (double)q.z + DM_DS * (3.0 - 4.0 * s / sm);
-      F[2 + cy][2 + cs] = hy * ((double)q.w + DM_DS * 4.0 * dm * s / (sm * sm));
+      F[cy][cs] = K + T + C + 3.0 * sig - 4.0 * log(sm);
+      F[2 + cy][cs] = hy * (Ky + Ty - 4.0 * dm / sm);
+      F[cy][2 + cs] = Ks + ds * (3.0 - 4.0 * s / sm);
+      F[2 + cy][2 + cs] = hy * (Kys + ds * 4.0 * dm * s / (sm * sm));
     }
   // coefficients A = H F H^T of the Hermite basis
   const double H[4][4] = {{1, 0, 0, 0}, {0, 0, 1, 0}, {-3, 3, -2, -1}, {2, -2, 1, 1}};
@@ -999,7 +1002,7 @@ void launch_master_to_planes(int64_t n, const float *master, const float *amax, 
 }
 
 // The distance-marginal table is a constant of the method, the same for every
-// context: it lives in this static device array (3.2 MB of nodes and 5.7 MB of cells, held by every GPU
+// context: it lives in this static device array (3.2 MB of nodes and 13.9 MB of cells, held by every GPU
 // that loads the library until the process exits) and is built once per CUDA
 // context of a device, by the first dotpe context created there, instead of
 // once per dotpe context.
