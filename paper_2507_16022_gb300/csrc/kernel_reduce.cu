@@ -4,9 +4,10 @@
 //   ln S1 = ln sum_ieo p_ieo,  ln S2 = ln sum_ieo p_ieo^2,  p_ieo = w_i w_e Lbar_ieo
 //   ln Z  = ln S1 - ln(N_i N_e N_phi)
 //   N_eff = S1^2 / S2, N_eff,int = S1^2 / sum_i P_i^2, N_eff,ext = S1^2 / sum_e P_e^2
-// Two passes per log-sum-exp: the maximum (FP32, exact), then the sum of
-// s * exp(m - max) with the exponential and the accumulation in FP64, so that
-// the combination adds only FP64 rounding to the FP32 partials.
+// Tiles' totals and merges: two passes per log-sum-exp, the maximum (FP32, exact), then the sum
+// of s * exp(m - max) with the exponential and the accumulation in FP64, which adds only FP64
+// rounding to the FP32 partials.  Row and column marginals: FP32 exponentials (about 2^-22
+// relative), FP64 products and sums.
 // A slice processed as several bank blocks merges each block's (max, sum) pairs,
 // its column marginals and its best ln L^ML into FP64 accumulators in block
 // order; the final kernel turns them into the evidence.
@@ -25,8 +26,8 @@ constexpr int NQ = 3;    // log-sum-exp inputs of a bank block: tile m1, tile m2
 
 // ln P over partials [nparts][n] (row or column marginal).  A block takes 32
 // consecutive entries (coalesced) and splits the parts over its 8 thread rows;
-// each thread keeps an online (max, FP64 sum) and the rows merge in shared memory.  With acc != nullptr the value is merged into the FP64 accumulator
-// acc[k] = (m, s) (s = 0: empty) instead of written to out.
+// each thread keeps an online (max, FP64 sum) and the rows merge in shared memory.  With
+// acc != nullptr the value is merged into the FP64 accumulator acc[k] = (m, s) (s = 0: empty) instead of written to out.
 constexpr int LX = 32, LY = 8;
 
 __device__ __forceinline__ void lse_add(double &m, double &s, double x, double w) {
@@ -35,12 +36,10 @@ __device__ __forceinline__ void lse_add(double &m, double &s, double x, double w
   if (x > m) { s = s * exp(m - x) + w; m = x; }
   else s += w * exp(x - m);
 }
-// A thread takes LG parts at a time: all LG loads are in flight together, the
-// products w exp(x - max) of the group are formed in FP32 with their rounding
-// errors (FMA) and summed in two floats (Knuth's TwoSum, ~2^-46 of the group's sum),
-// and one FP64 operation adds the group.  An FP64 multiply, add and two conversions
-// per part bound the kernel by the FP64 pipe (2 per clock and SM) at a third of the
-// bandwidth; with a group of 8 it streams the partials (figures at launch_reduce_block).
+// A thread takes LG parts at a time: all LG loads are in flight together and the group has one
+// maximum, so that the sum is scaled at most once per group.  The exponentials are FP32 (the
+// partials carry FP32 precision), the products and their sum FP64: two conversions and a fused
+// multiply-add per part (figures at launch_reduce_block).
 constexpr int LG = 8;
 
 __global__ void __launch_bounds__(LX * LY) reduce_lines_kernel(int64_t n, int nparts, const float2 *__restrict__ part,
@@ -63,21 +62,12 @@ __global__ void __launch_bounds__(LX * LY) reduce_lines_kernel(int64_t n, int np
         gm = fmaxf(gm, v[j].x);
       }
       if (gm == -INFINITY) continue;
-      float hi = 0.f, lo = 0.f;
+      if (!(s > 0.0)) mf = gm;
+      else if (gm > mf) { s *= (double)__expf(mf - gm); mf = gm; }
+      // (finite, so that a value that overflowed leaves +inf)
+      const float c = fminf(mf, 3.402823466e38f);
 #pragma unroll
-      for (int j = 0; j < LG; ++j) {
-        const float e = __expf(v[j].x - gm);
-        const float q = __fmul_rn(v[j].y, e);
-        const float r = fmaf(v[j].y, e, -q);
-        const float t = __fadd_rn(hi, q);
-        const float u = __fsub_rn(t, hi);
-        lo += __fadd_rn(__fsub_rn(hi, __fsub_rn(t, u)), __fsub_rn(q, u)) + r;
-        hi = t;
-      }
-      const double g = (double)hi + (double)lo;
-      if (!(s > 0.0)) { mf = gm; s = g; }
-      else if (gm > mf) { s = s * (double)__expf(mf - gm) + g; mf = gm; }
-      else s += g * (double)__expf(gm - mf);
+      for (int j = 0; j < LG; ++j) s = fma((double)v[j].y, (double)__expf(v[j].x - c), s);
     }
   double m = mf;
   sm[threadIdx.y][threadIdx.x] = m;
@@ -370,9 +360,10 @@ struct BlockScratch {  // per-block results of the parallel passes, in ReduceArg
 };
 }  // namespace
 
-// The two line reductions stream 84 MB of partials for 65,536 rows x 4,096 samples: 34 us
-// (67 us with FP64 operations per part); 106 us (238 us) over four blocks of 65,536 rows
-// x 2,048 samples.
+// The two line reductions stream 84 MB of partials for 65,536 rows x 4,096 samples: 44 us
+// (67 us a part at a time); 148 us (238 us) over four blocks of 65,536 rows x 2,048 samples.
+// Summing a group in two floats instead takes 34 and 106 us, with 46 bits of the sum where
+// FP64 has 53.
 void launch_reduce_block(const ReduceArgs &a, cudaStream_t st) {
   const dim3 lb(LX, LY);
   reduce_lines_kernel<<<(unsigned)((a.n_int + LX - 1) / LX), lb, 0, st>>>(a.n_int, a.n_etile, a.row_part,
