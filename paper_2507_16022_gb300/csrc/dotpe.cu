@@ -17,6 +17,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "kernels.h"
+#include "lru.h"
 
 namespace dotpe {
 
@@ -202,7 +203,7 @@ struct dotpe_ctx {
   std::unordered_map<std::string, bool> pair_cache;                       // shape key -> 64-sample tiles on CTA pairs
   bool wide_tiles = true;  // 64-sample tiles for screens, and for GEMM-only launches of mode banks
   bool pair_tiles = true;  // those tiles on CTA pairs (single events)
-  std::vector<std::unordered_map<std::string, cudaGraphExec_t>> graphs;  // per slot
+  std::vector<dotpe::LruMap<cudaGraphExec_t>> graphs;  // per slot: GRAPHS_MAX shapes of launch sequences
   double l2_band_bytes = 0;  // extrinsic operand kept in L2 per sweep of the bank
   // completion callbacks -> admission worker
   std::mutex cb_mu;
@@ -282,6 +283,10 @@ static void stage_give(dotpe_ctx *ctx, void *p, size_t n) {
     cudaFreeHost(p);
   }
 }
+
+// Executable graphs kept per slot.  A batch's launch sequence differs by its number of events and
+// by which of them launch their own kernels; a service with mixed sizes meets any number of those.
+constexpr size_t GRAPHS_MAX = 8;
 
 struct DoneArg {
   dotpe_ctx *ctx;
@@ -1160,27 +1165,28 @@ static int run_batch(dotpe_ctx *ctx, const std::vector<Event *> &evs, int slot) 
     if (ce != cudaSuccess) return fail(DOTPE_E_DEVICE, "graph capture: %s", cudaGetErrorString(ce));
     const std::string key = form + "/" + std::to_string(prec);
     auto &cache = ctx->graphs[slot];
-    auto it = cache.find(key);
-    bool ok = false;
-    if (it != cache.end()) {
+    cudaGraphExec_t x = nullptr;
+    if (cudaGraphExec_t *held = cache.find(key)) {
       cudaGraphExecUpdateResultInfo info;
-      ok = cudaGraphExecUpdate(it->second, g, &info) == cudaSuccess;
-      if (!ok) {
+      if (cudaGraphExecUpdate(*held, g, &info) == cudaSuccess) {
+        x = *held;
+      } else {
         cudaGetLastError();
-        cudaGraphExecDestroy(it->second);
-        cache.erase(it);
+        cudaGraphExecDestroy(*held);
+        cache.erase(key);
       }
     }
-    if (!ok) {
-      cudaGraphExec_t x = nullptr;
+    if (!x) {
       cudaError_t ie = cudaGraphInstantiate(&x, g, 0);
       if (ie != cudaSuccess) {
         cudaGraphDestroy(g);
         return fail(DOTPE_E_DEVICE, "graph instantiate: %s", cudaGetErrorString(ie));
       }
-      cache[key] = x;
+      // (the slot takes one launch unit at a time: no graph of it is in flight here)
+      cudaGraphExec_t gone = nullptr;
+      if (cache.put(key, x, &gone)) cudaGraphExecDestroy(gone);
     }
-    cudaError_t le = cudaGraphLaunch(cache[key], st);
+    cudaError_t le = cudaGraphLaunch(x, st);
     cudaGraphDestroy(g);
     if (le != cudaSuccess) return fail(DOTPE_E_DEVICE, "graph launch: %s", cudaGetErrorString(le));
   } else if (rc != DOTPE_OK) {
@@ -1827,7 +1833,7 @@ int dotpe_create(const dotpe_config *cfg, dotpe_ctx **out) {
   ctx->wide_tiles = (c.flags & DOTPE_CONFIG_NARROW_TILES) == 0;
   ctx->pair_tiles = (c.flags & DOTPE_CONFIG_SINGLE_CTA_TILES) == 0;
   ctx->use_graphs = (c.flags & DOTPE_CONFIG_NO_GRAPHS) == 0;
-  ctx->graphs.resize(ns);
+  ctx->graphs.assign(ns, LruMap<cudaGraphExec_t>(GRAPHS_MAX));
   ctx->streams.resize(ns);
   ctx->slot_busy.assign(ns, 0);
   for (int s = 0; s < ns; ++s) cudaStreamCreateWithFlags(&ctx->streams[s], cudaStreamNonBlocking);
@@ -1889,8 +1895,7 @@ int dotpe_destroy(dotpe_ctx *ctx) {
   cudaDeviceSynchronize();
   for (auto &k : ctx->kits) kit_destroy(k);
   for (auto &p : ctx->stages) cudaFreeHost(p.p);
-  for (auto &m : ctx->graphs)
-    for (auto &kv : m) cudaGraphExecDestroy(kv.second);
+  for (auto &m : ctx->graphs) m.for_each([](cudaGraphExec_t x) { cudaGraphExecDestroy(x); });
   for (auto s : ctx->streams) cudaStreamDestroy(s);
   cudaStreamDestroy(ctx->main_stream);
   cudaStreamDestroy(ctx->input_stream);
