@@ -652,7 +652,7 @@ static EpiParams refine_params(const EventRun &R) {
   return Pf;
 }
 
-static std::string band_key(const Event &e, const ScratchLayout &L, bool split);
+static std::string band_key(dotpe_ctx *ctx, const Event &e, const ScratchLayout &L);
 
 // Tile width of a single-pass launch: 64-sample tiles where the launch writes
 // no marginal partials (a screening pass with the cut on, or GEMM-only of a mode
@@ -668,17 +668,20 @@ static std::string band_key(const Event &e, const ScratchLayout &L, bool split);
 // 0.80 and 0.86 ms; 16,384 x 256, K = 1,024 (431 steps) 0.50 and 0.43; 2,048 x 512 (108
 // steps) 0.41 and 0.33; 300 x 77 0.34 and 0.23.
 constexpr int64_t POL_WIDE_STEPS = 1500;  // 128 x 32-pair tiles x modes x k-blocks of 64, per SM
-static bool wide_form(dotpe_ctx *ctx, const Event &e, const ScratchLayout &L, const EpiParams &P, bool split) {
-  if (!ctx->wide_tiles || split || P.lnl_tile) return false;
+static bool wide_form(dotpe_ctx *ctx, const Event &e, const ScratchLayout &L, int64_t n_int) {
+  // (a launch of split operands marginalises; stored values are written by 32-sample tiles)
+  const bool split = prec_split(e.prec) && e.prec != DOTPE_PREC_MIXED, gemm = (e.flags & DOTPE_FLAG_GEMM_ONLY) != 0;
+  const bool screen = e.prec == DOTPE_PREC_MIXED && e.cut > 0;
+  if (!ctx->wide_tiles || split || (e.flags & DOTPE_FLAG_STORE_LNL)) return false;
   const Bank &b = *e.bank;
-  if (b.n_pol != 2) return P.gemm_only || P.screen_ml;
-  if (P.gemm_only || !P.screen_ml || prec_bf16(e.prec)) return false;
-  const int64_t tiles = (P.n_int + TC_TI - 1) / TC_TI * L.n_etile;
+  if (b.n_pol != 2) return gemm || screen;
+  if (gemm || !screen) return false;
+  const int64_t tiles = (n_int + TC_TI - 1) / TC_TI * L.n_etile;
   return tiles * b.M * (b.Kpad / 64) >= POL_WIDE_STEPS * ctx->n_sms;
 }
-static int launch_tev(dotpe_ctx *ctx, const Event &e, const ScratchLayout &L, const EpiParams &P, bool split) {
-  if (!wide_form(ctx, e, L, P, split)) return 32;
-  auto it = ctx->tev_cache.find(band_key(e, L, prec_split(e.prec)));
+static int launch_tev(dotpe_ctx *ctx, const Event &e, const ScratchLayout &L, int64_t n_int) {
+  if (!wide_form(ctx, e, L, n_int)) return 32;
+  auto it = ctx->tev_cache.find(band_key(ctx, e, L));
   return it != ctx->tev_cache.end() ? it->second : 64;
 }
 
@@ -686,7 +689,7 @@ static int launch_tev(dotpe_ctx *ctx, const Event &e, const ScratchLayout &L, co
 // choice for the shape where it has one, else the context's default.
 static bool launch_pair(dotpe_ctx *ctx, const Event &e, const ScratchLayout &L) {
   if (!ctx->pair_tiles) return false;
-  auto it = ctx->pair_cache.find(band_key(e, L, prec_split(e.prec)));
+  auto it = ctx->pair_cache.find(band_key(ctx, e, L));
   return it != ctx->pair_cache.end() ? it->second : true;
 }
 
@@ -725,14 +728,14 @@ static int event_fused(dotpe_ctx *ctx, Event &e, EventRun &R, bool last_block, c
   TcWork W = R.W;
   if (!R.mixed) {
     W.P = R.P;
-    T.tev = launch_tev(ctx, e, R.L, W.P, T.split);
+    T.tev = launch_tev(ctx, e, R.L, W.P.n_int);
     T.pair = launch_pair(ctx, e, R.L);
     int r = launch_tc(T, &W, 1, nullptr, nullptr, st);
     if (r != 0) return fail(DOTPE_E_DEVICE, "tcgen05 kernel launch failed: %s", cudaGetErrorString((cudaError_t)r));
     return DOTPE_OK;
   }
   W.P = screen_params(R);
-  T.tev = launch_tev(ctx, e, R.L, W.P, false);
+  T.tev = launch_tev(ctx, e, R.L, W.P.n_int);
   T.pair = launch_pair(ctx, e, R.L);
   if (T.tev == 64 && (rc = hh_bound_pass(ctx, e, R, W.P, st)) != DOTPE_OK) return rc;
   int r = launch_tc(T, &W, 1, nullptr, nullptr, st);
@@ -932,18 +935,21 @@ static int run_event(dotpe_ctx *ctx, Event &e) {
 // 64-sample tiles run on CTA pairs (cta_group::2, M = 256: each SM loads half
 // of the tile's extrinsic rows) or on one SM each on how the mainloop's
 // shared-memory ingress weighs against the pair's tail; all three are chosen
-// per shape (precision class, modes, k-blocks, extrinsic tiles) by timing
+// per shape (band_key) by timing
 // candidates on the first event of that shape.
 // ---------------------------------------------------------------------------
-static std::string band_key(const Event &e, const ScratchLayout &L, bool split) {
+// The shape that a choice is made for.  Whether its launches may take 64-sample tiles at all is
+// part of it: an event that may not (stored values, no cut, a small polarisation-resolved one)
+// has other candidates, and its choice must not become that of the events that may.
+static std::string band_key(dotpe_ctx *ctx, const Event &e, const ScratchLayout &L) {
   char buf[96];
-  snprintf(buf, sizeof(buf), "%d/%d/%d/%d/%d", prec_bf16(e.prec) ? 1 : 0, split ? 1 : 0, e.bank->M, e.bank->Kpad,
-           L.n_etile);
+  snprintf(buf, sizeof(buf), "%d/%d/%d/%d/%d/%d/%d", prec_bf16(e.prec) ? 1 : 0, prec_split(e.prec) ? 1 : 0,
+           e.bank->M, e.bank->n_pol, e.bank->Kpad, L.n_etile, wide_form(ctx, e, L, L.block_rows) ? 1 : 0);
   return buf;
 }
 
 static int event_band(dotpe_ctx *ctx, const Event &e, const ScratchLayout &L, bool split) {
-  auto it = ctx->band_cache.find(band_key(e, L, split));
+  auto it = ctx->band_cache.find(band_key(ctx, e, L));
   if (it != ctx->band_cache.end()) return std::min(it->second, L.n_etile);
   return tc_band(ctx->l2_band_bytes, e.bank->Kpad / 64, e.bank->M, split, L.n_etile);
 }
@@ -956,7 +962,7 @@ static int event_band(dotpe_ctx *ctx, const Event &e, const ScratchLayout &L, bo
 // launch that follows.  Blocks the calling thread once per shape.
 static int autotune_band(dotpe_ctx *ctx, Event &e, EventRun &R, cudaStream_t st) {
   const bool split_main = prec_split(e.prec) && e.prec != DOTPE_PREC_MIXED;
-  const std::string key = band_key(e, R.L, prec_split(e.prec));
+  const std::string key = band_key(ctx, e, R.L);
   if (e.prec == DOTPE_PREC_FP32 || ctx->band_cache.count(key)) return DOTPE_OK;
   TcLaunch T;
   int rc = tc_launch_of(ctx, *e.bank, e.prec, T);
@@ -966,7 +972,7 @@ static int autotune_band(dotpe_ctx *ctx, Event &e, EventRun &R, cudaStream_t st)
   TcWork W = R.W;
   W.P = R.mixed ? screen_params(R) : R.P;
   std::vector<int> tevs{32};
-  if (wide_form(ctx, e, R.L, W.P, split_main)) tevs.push_back(64);
+  if (wide_form(ctx, e, R.L, W.P.n_int)) tevs.push_back(64);
   // the 64-sample candidates timed as they run: with the <h|h> bound where the event has it
   if (R.mixed && tevs.back() == 64 && (rc = hh_bound_pass(ctx, e, R, W.P, st)) != DOTPE_OK) return rc;
   const int dflt = tc_band(ctx->l2_band_bytes, e.bank->Kpad / 64, e.bank->M, prec_split(e.prec), R.L.n_etile);
@@ -1099,7 +1105,7 @@ static int run_batch(dotpe_ctx *ctx, const std::vector<Event *> &evs, int slot) 
         // one tile width for the launch: 64 samples only if every event takes it
         T1.tev = 64;
         for (int k = k0; k < k0 + m; ++k)
-          T1.tev = std::min(T1.tev, launch_tev(ctx, *evs[shared[k]], R[shared[k]].L, W[k].P, T1.split));
+          T1.tev = std::min(T1.tev, launch_tev(ctx, *evs[shared[k]], R[shared[k]].L, W[k].P.n_int));
         if (mixed && T1.tev == 64)
           for (int k = k0; k < k0 + m; ++k) {
             int rb = hh_bound_pass(ctx, *evs[shared[k]], R[shared[k]], W[k].P, st);
