@@ -1242,6 +1242,8 @@ static void progress(dotpe_ctx *ctx) {
       } else if (q != cudaErrorNotReady) {
         cudaGetLastError();
         e.state = DOTPE_STATE_FAILED;
+        e.launch_error = cudaGetErrorString(q);
+        if (e.h_out->status == STATUS_PENDING) e.h_out->status = 0;  // (no device status)
         ctx->slot_busy[e.slot]--;
       }
     }
