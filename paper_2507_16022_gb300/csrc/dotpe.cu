@@ -1088,6 +1088,7 @@ static int run_batch(dotpe_ctx *ctx, const std::vector<Event *> &evs, int slot) 
     for (int k : own) {
       int r = event_fused(ctx, *evs[k], R[k], true, st);
       if (r != DOTPE_OK) return r;
+      CUDA_OR_FAIL(record(evs[k]->ev_k1, st));
     }
     const int ns = (int)shared.size();
     if (ns > 0) {
@@ -1151,8 +1152,8 @@ static int run_batch(dotpe_ctx *ctx, const std::vector<Event *> &evs, int slot) 
         }
       }
     }
+    for (int k : shared) CUDA_OR_FAIL(record(evs[k]->ev_k1, st));
     for (int k = 0; k < n; ++k) {
-      CUDA_OR_FAIL(record(evs[k]->ev_k1, st));
       R[k].ra.first = 1;
       launch_reduce_block(R[k].ra, st);
       int r = event_end(ctx, *evs[k], R[k], st);
