@@ -249,11 +249,11 @@ __device__ __forceinline__ void phase_quad(const float (&Zr)[4], const float (&Z
   const float h2 = fmaf(Cr[1], e.z, -Ci[1] * e.w);
   const float hr = fmaf(Cr[0], e.x, fmaf(-Ci[0], e.y, fmaf(Cr[2], f.x, -Ci[2] * f.y)));
   const float hi = fmaf(Cr[2], f.y, fmaf(Ci[2], f.x, -fmaf(Cr[0], e.y, Ci[0] * e.x)));
-  const float hp = fmaf(2.f, h2, C0), hm = fmaf(-2.f, h2, C0);
-  hh[0] = fmaf(2.f, hr, hp);
-  hh[1] = fmaf(2.f, hi, hm);
-  hh[2] = fmaf(-2.f, hr, hp);
-  hh[3] = fmaf(-2.f, hi, hm);
+  // (one rounding at the size of C_0, as in phase_at: the sums of the other terms are smaller)
+  hh[0] = fmaf(2.f, h2 + hr, C0);
+  hh[1] = fmaf(2.f, hi - h2, C0);
+  hh[2] = fmaf(2.f, h2 - hr, C0);
+  hh[3] = fmaf(-2.f, h2 + hi, C0);
 }
 
 __device__ __forceinline__ float lnl_ml_of(float dh, float hh) {
