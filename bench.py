@@ -72,7 +72,7 @@ CUT_DELTA = 20.0  # Eq. coherent_ML_selection, the paper's value
 # capture of the DRAM counters at the workload's own size (the bound's 2 bytes
 # per pair stay in L2 at small sizes, so a small capture does not scale):
 # the shape it was taken on.  None = no capture of the current kernels.
-SCREEN_TRAFFIC = {"bytes": 0.504e9 + 6.398e9, "n_int": 65536, "n_ext": 4096,
+SCREEN_TRAFFIC = {"bytes": 0.507e9 + 6.176e9, "n_int": 65536, "n_ext": 4096,
                   "source": "profiles/launch_lists.md"}
 
 

@@ -2768,22 +2768,23 @@ int dotpe_lnl_blocks(dotpe_ctx *ctx, uint64_t event_id, int64_t i0, int64_t i1, 
     const bool row = what == DOTPE_ROW_MARGINAL;
     int64_t a = row ? i0 : e0, z = row ? i1 : e1, n = row ? e.NI : e.NE;
     if (a < 0 || z > n || z <= a) return fail(DOTPE_E_INVALID, "marginal range");
-    if (is_device_ptr(out)) {
-      // Converted into a buffer of the context's device and copied from there, on the default
-      // stream: `out` may be another device's or managed memory, or not aligned to a float, which
-      // a copy takes and a kernel's stores do not.
-      const size_t bytes = (size_t)(z - a) * sizeof(float);
-      float *tmp = nullptr;
-      CUDA_OR_FAIL(cudaMallocAsync((void **)&tmp, bytes, 0));
-      launch_to_float(z - a, (row ? e.ln_p_int : e.ln_p_ext) + a, tmp, 0);
+    // To device memory: converted into a buffer of the context's device and copied from there, on
+    // the default stream.  `out` may be another device's or managed memory, or not aligned to a
+    // float, which a copy takes and a kernel's stores do not.  (Without room for the buffer, as to
+    // the host.)
+    const size_t bytes = (size_t)(z - a) * sizeof(float);
+    float *buf = nullptr;
+    if (is_device_ptr(out) && cudaMallocAsync((void **)&buf, bytes, 0) == cudaSuccess) {
+      launch_to_float(z - a, (row ? e.ln_p_int : e.ln_p_ext) + a, buf, 0);
       cudaError_t ce = cudaGetLastError();
-      if (ce == cudaSuccess) ce = cudaMemcpyAsync(out, tmp, bytes, cudaMemcpyDefault, 0);
-      cudaFreeAsync(tmp, 0);
+      if (ce == cudaSuccess) ce = cudaMemcpyAsync(out, buf, bytes, cudaMemcpyDefault, 0);
+      cudaFreeAsync(buf, 0);
       const cudaError_t se = cudaStreamSynchronize(0);
       CUDA_OR_FAIL(ce);
       CUDA_OR_FAIL(se);
       return DOTPE_OK;
     }
+    cudaGetLastError();
     std::vector<double> tmp(z - a);
     CUDA_OR_FAIL(cudaMemcpy(tmp.data(), (row ? e.ln_p_int : e.ln_p_ext) + a, (z - a) * 8, cudaMemcpyDeviceToHost));
     std::vector<float> f(z - a);

@@ -13,7 +13,7 @@
 // a thread reads 8 + 8 times 16 bytes for 128 packed FMAs, every read one wavefront (rows 20
 // and samples 36 words apart), so shared memory is half busy and the FMA pipe is what is
 // left: 8,192 x 1,024, B 512, M 4 takes 2.6 ms without the epilogue (1.85 ms at the pipe's
-// rate), 2.8 ms with it and 3.1 ms with every pair stored.  It was 4.5 ms with every mode in each
+// rate), 2.8 ms with it and 3.3 ms with every pair stored under a cut.  It was 4.5 ms with every mode in each
 // thread (4 rows x 2 samples, shared memory 78% busy).  Measured and not kept: scalar FMAs
 // (3.7 ms), 4 rows x 8 samples (3.3 ms), sums split into even and odd k so that the
 // operands need no copy of the row's value into both halves (4 x 4 per thread, 3.7 ms).

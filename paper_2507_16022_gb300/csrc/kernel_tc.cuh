@@ -53,9 +53,9 @@ namespace {
 constexpr int TI = TC_TI, TE = TC_TE, BK = 64;
 // Epilogue warps: 8 for the screens (168 registers, row records in registers), 16 for the
 // marginalising kernels (96 registers), whose table gathers and 32-phase loops are latency:
-// 12,289 rows x 771 samples without a cut (fp16x3) take 3.8 ms, 11.9 ms before with 8
+// 12,289 rows x 771 samples without a cut (fp16x3) take 4.2 ms, 11.9 ms before with 8
 // warps, erfc / erfcx per phase and the node table; the refinement of 32,768 x 2,048
-// concentrated pairs 3.9 ms (5.2 ms), 2.85 ms of it its loads and MMAs alone.
+// concentrated pairs 4.6 ms (5.2 ms), 2.85 ms of it its loads and MMAs alone.
 __host__ __device__ constexpr int epi_warps(int tev, bool scr) { return tev == 32 && !scr ? 16 : 8; }
 __host__ __device__ constexpr int cta_threads(int tev, bool scr) { return (2 + epi_warps(tev, scr)) * 32; }
 constexpr uint32_t A_BYTES = TI * BK * 2;  // one k-block of the bank tile
