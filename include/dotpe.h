@@ -403,8 +403,8 @@ int dotpe_event_submit(dotpe_ctx *ctx, const dotpe_event_desc *desc, uint64_t *e
  * one event after the other (mixed precision: one screening launch, one
  * selection over them, one refinement launch), then every event's reduction.  The
  * sequence is captured as a CUDA graph (unless DOTPE_CONFIG_NO_GRAPHS) whose
- * executable is kept per slot and updated in place for the next batch.  Each
- * event's results are those it gets when submitted alone (same tiles, same
+ * executable is kept per slot (for the eight shapes of sequence used last) and
+ * updated in place for the next batch of its shape.  Each event's results are those it gets when submitted alone (same tiles, same
  * per-event reductions).  descs[k].block_rows must be 0.  event_ids: [n] out.
  * The paper has no counterpart (it evaluates one event at a time, Sec. IV).
  * Errors: as dotpe_event_submit for any event (then none is queued);
